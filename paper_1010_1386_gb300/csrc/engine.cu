@@ -18,16 +18,20 @@ thread_local std::string g_err;
 constexpr size_t kAlign = 256;
 size_t align_up(size_t x) { return (x + kAlign - 1) & ~(kAlign - 1); }
 
-// Normal-sequence coefficient updates of the remainder sequence (a4 count).
-double prs_updates(int a, int b) {
+// Modular products of the normal remainder sequence (a4 count): three per
+// coefficient of a double step, two of the single step between equal degrees.
+double prs_products(int a, int b) {
   double u = 0;
   while (a > 0 && b > 0) {
-    if (a >= b) {
-      u += a;
+    if (a == b) {
+      u += 2.0 * a;
       --a;
+    } else if (a > b) {
+      u += 3.0 * (a - 1);
+      a -= 2;
     } else {
-      u += b;
-      --b;
+      u += 3.0 * (b - 1);
+      b -= 2;
     }
   }
   return u;
@@ -526,7 +530,7 @@ int rs_build_batch(rs_ctx *ctx, int n, const rs_bipoly *f, const rs_bipoly *g,
       b->info.modmul_prs += imgs * 4.0 * r * (r + 1.0);
     } else {
       b->info.modmul_eval += imgs * (0.5 * (p.f.nc + p.g.nc) + (p.f.my + 1) + (p.g.my + 1));
-      b->info.modmul_prs += imgs * 2.0 * prs_updates(p.f.my, p.g.my);
+      b->info.modmul_prs += imgs * prs_products(p.f.my, p.g.my);
     }
     b->info.modmul_interp += (double)p.K * ((double)d.NI * d.NI / 2 + 8.0 * d.NI);  // two interpolations of NI / 2
     b->info.modmul_crt += (double)p.N * ((double)d.K * (d.K - 1) + d.K);

@@ -26,27 +26,66 @@
 //   Res_{0,b}(A,B) = A_0^b,  Res_{a,0}(A,B) = B_0^a
 //
 // (each identity is a row operation on the Sylvester matrix followed by a
-// cofactor expansion along its first column).  The pivot powers
-// prod_t c_t^{e_t}, e_t = deg(pivot_t) - 1, are non-increasing in t, so they
-// are accumulated by Abel summation: with Q_t = c_1 ... c_t,
-// prod_t c_t^{e_t} = prod_t Q_t^{e_t - e_{t+1}}: one product per step into Q
-// and one into the denominator whenever e drops.
+// cofactor expansion along its first column).  Two steps in a row reduce the
+// same polynomial whenever a >= b + 1 (pivot l_B twice), and they are taken in
+// one pass over its coefficients:
+//
+//   a >= b + 1, l_B != 0:  A'' = l_B^2 A - (alpha y + beta) y^(a-b-1) B,
+//     alpha = l_B A_0, beta = l_B A_1 - A_0 B_1 (index = power below the top);
+//     Res_{a,b}(A,B) (l_B^2)^{b-1} = Res_{a-2,b}(A'',B), and the same on B.
+//
+// In the normal sequence (degrees one apart) every pass is of this kind: three
+// products and one Montgomery reduction per coefficient for two degrees,
+// against four products and two reductions in single steps.  The three
+// multipliers c (each below p) are negated together when their sum exceeds
+// 2^32, so that their products with residues stay below 2^32 p and one
+// unsigned REDC finishes the sum; a pass on A negated so gives
+// (-1)^b Res(A'', B).
+//
+// The pivot powers prod_t c_t^{e_t} (c the pivot of a single step, e its
+// degree minus one; the square of the pivot in a double step) have
+// non-increasing e_t, so they are accumulated by Abel summation: with
+// Q_t = c_1 ... c_t, prod_t c_t^{e_t} = prod_t Q_t^{e_t - e_{t+1}}: one product
+// per pass into Q and one into the denominator whenever e drops.
 //
 // Register arrays have a compile-time capacity C; once both degrees fit in
-// C - 8 entries the state moves to arrays of C - 8 (registers are renamed,
-// nothing is copied), so the unrolled update loops shrink with the degrees.
+// C - S entries (S = RS_G1_PSTEP) the state moves to arrays of C - S (registers
+// are renamed, nothing is copied), so the unrolled update loops shrink with
+// the degrees.
+//
+// Bound: the multiply pipe.  A wide product costs 4.2 issue cycles per warp
+// and SM partition, a low one 2.1: 19.5 cycles per coefficient of a double
+// pass against 2 x 15.2 in single steps (both measured with 16 warps per SM
+// on arrays of 24).  G1 on batches of 16 pairs with deg_x = 24, 32-bit
+// coefficients, ns per image with single and with double steps:
+//   deg_y       14     22     28     38     44     52     60     68
+//   single   0.305  0.460  0.653  0.998  1.302  1.756  2.297  2.550
+//   double   0.284  0.404  0.578  0.817  1.075  1.389  1.802  2.081
+// (the evaluation is in both).
 #include "rs_internal.cuh"
 
+// Register capacity dropped per phase (S), entries per length check of a
+// double step (T) and minimum resident 128-thread blocks per SM requested from
+// ptxas (caps registers at 65536 / (128 * MINB) per thread), per capacity C.
+// A phase costs code (two unrolled double steps; with many phases the warps
+// miss the instruction cache: at C = 56 "no instruction" took 19% of the
+// stalls with S = 12, 7% with 28), a longer phase more length checks.
+// ns per image, deg_y = C - 4 (C - 2 at 16, 24 and 40):
+//   C                    16     24     32     40     48     56     64     72
+//   S = 12, T = 2     0.289  0.426  0.573  0.886  1.152  1.503  2.006  2.098
+//   S = 16, T = 2     0.282  0.438  0.562  0.849  1.099  1.459  1.899  2.113
+//   S = 20, T = 4     0.288  0.415  0.569  0.815  1.097  1.412  1.844  2.103
+//   S = 28, T = 4     0.292  0.416  0.573  0.846  1.075  1.386  1.795  2.110
+//   5 blocks, S = 12  0.291  0.402  0.571  0.909  1.251
 #ifndef RS_G1_PSTEP
-#define RS_G1_PSTEP 12  // register capacity dropped per phase
+#define RS_G1_PSTEP (RS_G1_CAP <= 8 ? 8 : RS_G1_CAP <= 16 ? 16 : RS_G1_CAP <= 24 ? 12 : RS_G1_CAP <= 32 ? 16 \
+                     : RS_G1_CAP <= 40 ? 20 : RS_G1_CAP <= 64 ? 28 : 12)
 #endif
-// Minimum resident 128-thread blocks per SM requested from ptxas per register
-// capacity (caps registers at 65536 / (128 * MINB) per thread).
-#if defined(RS_G1_MINB_AT) && defined(RS_G1_MINB_SET) && RS_G1_MINB_AT == RS_G1_CAP
-#define RS_G1_MINB RS_G1_MINB_SET  // tuning override for one capacity
+#ifndef RS_G1_TAIL
+#define RS_G1_TAIL (RS_G1_CAP <= 32 || RS_G1_CAP > 64 ? 2 : 4)
 #endif
 #ifndef RS_G1_MINB
-#define RS_G1_MINB (RS_G1_CAP <= 24 ? 6 : RS_G1_CAP <= 48 ? 4 : 3)
+#define RS_G1_MINB (RS_G1_CAP <= 16 ? 6 : RS_G1_CAP <= 24 ? 5 : RS_G1_CAP <= 48 ? 4 : 3)
 #endif
 
 namespace {
@@ -90,8 +129,8 @@ __device__ __forceinline__ void reduce_tail(uint32_t (&P)[C], const uint32_t (&V
 
 // P[i] <- w1 P[i+1] + w2 V[i+1] for i < live (the reduced polynomial's
 // entries); the top entry (which cancels) is dropped.  Every caller reduces
-// an array whose degree is at least C - 8 (the phase condition), so the
-// first C - 8 entries are always live and only the last 7 are checked.
+// an array whose degree is at least C - S (the phase condition), so the
+// first C - S entries are always live and only the last S - 1 are checked.
 template <int C>
 __device__ __forceinline__ void reduce_into(uint32_t (&P)[C], const uint32_t (&V)[C], uint32_t w1,
                                             uint32_t w2, const ModP &m, int live) {
@@ -102,6 +141,53 @@ __device__ __forceinline__ void reduce_into(uint32_t (&P)[C], const uint32_t (&V
   P[C - 1] = 0u;
 }
 
+// Entry I of a double step.
+template <int C, int I>
+__device__ __forceinline__ void reduce2_entry(uint32_t (&P)[C], const uint32_t (&V)[C], uint32_t c2, uint32_t c1,
+                                              uint32_t c0, const ModP &m) {
+  if constexpr (I < C - 2)
+    P[I] = redc((uint64_t)P[I + 2] * c2 + (uint64_t)V[I + 2] * c1 + (uint64_t)V[I + 1] * c0, m.p, m.pinv);
+  else if constexpr (I < C)
+    P[I] = 0u;
+}
+
+template <int C, int I, int E>
+__device__ __forceinline__ void reduce2_entries(uint32_t (&P)[C], const uint32_t (&V)[C], uint32_t c2, uint32_t c1,
+                                                uint32_t c0, const ModP &m) {
+  if constexpr (I < E) {
+    reduce2_entry<C, I>(P, V, c2, c1, c0, m);
+    reduce2_entries<C, I + 1, E>(P, V, c2, c1, c0, m);
+  }
+}
+
+// Entries I .. C - 1 of a double step whose result has `live` entries, in
+// groups; a group that is not computed holds only the two entries shifted
+// out, which become zero (computed entries past the length come out zero).
+template <int C, int I>
+__device__ __forceinline__ void reduce2_tail(uint32_t (&P)[C], const uint32_t (&V)[C], uint32_t c2, uint32_t c1,
+                                             uint32_t c0, const ModP &m, int live) {
+  if constexpr (I < C) {
+    if (live > I) {
+      reduce2_entries<C, I, I + RS_G1_TAIL>(P, V, c2, c1, c0, m);
+      reduce2_tail<C, I + RS_G1_TAIL>(P, V, c2, c1, c0, m, live);
+    } else {
+      P[I] = 0u;
+      if constexpr (I + 1 < C) P[I + 1] = 0u;
+    }
+  }
+}
+
+// P[i] <- c2 P[i+2] + c1 V[i+2] + c0 V[i+1] for i < live: two steps on P, the
+// two top entries (which cancel) dropped.  c2 + c1 + c0 <= 2^32.  Callers
+// reduce a degree of at least C - S (S the phase), so live >= C - S - 1.
+template <int C>
+__device__ __forceinline__ void reduce2_into(uint32_t (&P)[C], const uint32_t (&V)[C], uint32_t c2, uint32_t c1,
+                                             uint32_t c0, const ModP &m, int live) {
+  constexpr int H = C > RS_G1_PSTEP ? C - RS_G1_PSTEP - 1 : 0;
+  reduce2_entries<C, 0, H>(P, V, c2, c1, c0, m);
+  reduce2_tail<C, H>(P, V, c2, c1, c0, m, live);
+}
+
 template <int C>
 __device__ __forceinline__ void drop_top(uint32_t (&P)[C]) {
 #pragma unroll
@@ -109,7 +195,7 @@ __device__ __forceinline__ void drop_top(uint32_t (&P)[C]) {
   P[C - 1] = 0u;
 }
 
-// One normal step on A (a >= b, l_B != 0) or on B (a < b, l_A != 0).
+// One normal step on A (a >= b, l_B != 0).
 template <int C>
 __device__ __forceinline__ void step_a(uint32_t (&A)[C], const uint32_t (&B)[C], Prs &s, const ModP &m) {
   const uint32_t lb = B[0], la = A[0];
@@ -119,27 +205,52 @@ __device__ __forceinline__ void step_a(uint32_t (&A)[C], const uint32_t (&B)[C],
   --s.a;
 }
 
+// Two steps at once on P (formal degree d, reduced) with V (formal degree
+// e <= d - 1, pivot V[0] != 0): returns 1 if the result was negated.
 template <int C>
-__device__ __forceinline__ void step_b(const uint32_t (&A)[C], uint32_t (&B)[C], Prs &s, const ModP &m) {
-  const uint32_t la = A[0], lb = B[0];
-  settle(s, s.a - 1, la, m);
-  reduce_into<C>(B, A, la, mneg(lb, m.p), m, s.b);
-  --s.b;
+__device__ __forceinline__ uint32_t step2(uint32_t (&P)[C], const uint32_t (&V)[C], int d, int e, Prs &s,
+                                          const ModP &m) {
+  const uint32_t lv = V[0], np0 = m.p - P[0];  // in (0, p]
+  uint32_t c2 = mmul(lv, lv, m);
+  settle(s, e - 1, c2, m);
+  uint32_t c1 = mmul(lv, np0, m);                         // -lv P_0
+  uint32_t c0 = mmul2(P[0], V[1], m.p - lv, P[1], m);     // P_0 V_1 - lv P_1
+  // halves: a sum below 2^31 - 1 bounds c2 + c1 + c0 by 2^32 - 1; otherwise
+  // the negated sum is at most 3 p - (2^32 - 2) < 2^31 + 2
+  const uint32_t neg = (c2 >> 1) + (c1 >> 1) + (c0 >> 1) >= 0x7fffffffu ? 1u : 0u;
+  if (neg) {
+    c2 = m.p - c2;
+    c1 = m.p - c1;
+    c0 = m.p - c0;
+  }
+  reduce2_into<C>(P, V, c2, c1, c0, m, d - 1);
+  return neg;
 }
 
 template <int C>
 __device__ __forceinline__ void prs_run(uint32_t (&A)[C], uint32_t (&B)[C], Prs &s, const ModP &m) {
   // invariant: a, b <= C - 1
   constexpr int S = RS_G1_PSTEP;
-  // Fast path for the normal sequence, with a fixed role for each array in
-  // every loop (no data-dependent choice of which array to update): first
-  // reduce the larger degree down to the smaller, then alternate A, B.
-  while (s.a > s.b && s.b > 0 && B[0] != 0u && (C <= S || s.a > C - S - 1)) step_a<C>(A, B, s, m);
-  while (s.b > s.a && s.a > 0 && A[0] != 0u && (C <= S || s.b > C - S - 1)) step_b<C>(A, B, s, m);
-  while (s.a == s.b && s.a > 1 && B[0] != 0u && (C <= S || s.a > C - S - 1)) {
-    step_a<C>(A, B, s, m);  // (a, a) -> (a - 1, a)
-    if (A[0] == 0u) break;
-    step_b<C>(A, B, s, m);  // (a - 1, a) -> (a - 1, a - 1)
+  // Fast path: double steps on the polynomial of larger degree (after one
+  // single step if the degrees are equal), until a pivot vanishes or both
+  // degrees fit the next phase.
+  for (;;) {
+    if (s.a == s.b) {
+      if (s.a < 1 || B[0] == 0u || (C > S && s.a <= C - S - 1)) break;
+      step_a<C>(A, B, s, m);
+    }
+    if (s.b > s.a) {
+      if (s.a < 1 || A[0] == 0u || (C > S && s.b <= C - S - 1)) break;
+      const uint32_t neg = step2<C>(B, A, s.b, s.a, s, m);
+      s.sign ^= neg & (uint32_t)s.a;
+      s.b -= 2;
+    }
+    if (s.a > s.b) {
+      if (s.b < 1 || B[0] == 0u || (C > S && s.a <= C - S - 1)) break;
+      const uint32_t neg = step2<C>(A, B, s.a, s.b, s, m);
+      s.sign ^= neg & (uint32_t)s.b;
+      s.a -= 2;
+    }
   }
   // General steps: zero pivots, the last steps, and the phase boundary.
   while (s.a > 0 && s.b > 0 && (C <= S || s.a > C - S - 1 || s.b > C - S - 1)) {
