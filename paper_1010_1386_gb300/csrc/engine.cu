@@ -579,7 +579,11 @@ int rs_build_batch(rs_ctx *ctx, int n, const rs_bipoly *f, const rs_bipoly *g,
     }
     ch.persistent = (ch.persistent && opt.persistent) ? 1 : 0;
     if (opt.g1_threads > 0 || ctx->cfg.tile_points > 0) ch.persistent = opt.persistent ? 1 : 0;
-    const int T = ch.threads;
+    // The per-thread columns and the staged coefficients of the largest accepted
+    // inputs exceed a block's shared memory with 128 threads at C = 72.
+    int T = ch.threads;
+    for (int i : members)
+      while (T > 32 && rs_g1_smem_words(b->plans[i], cap, T) * 4 > RS_G1_MAX_SMEM_BYTES) T >>= 1;
     RsClassLaunch cl;
     cl.cap = cap;
     cl.threads = T;
@@ -595,7 +599,7 @@ int rs_build_batch(rs_ctx *ctx, int n, const rs_bipoly *f, const rs_bipoly *g,
     for (int i : members) {
       const PairPlan &p = b->plans[i];
       cl.cost += (double)p.K * p.N * (p.f.nc + p.g.nc + 2.0 * p.f.my * p.g.my);
-      cl.smem = std::max(cl.smem, (size_t)rs_g1_staged_words(p, cap, T) * 4);
+      cl.smem = std::max(cl.smem, (size_t)rs_g1_smem_words(p, cap, T) * 4);
       const int M = (p.N + 1) / 2;  // point pairs: two threads each
       for (int k = 0; k < p.K; ++k) {
         if (ctx->cfg.univariate == 0) {

@@ -326,83 +326,119 @@ __device__ __forceinline__ int32_t signed_rep(uint32_t v, uint32_t p) {
 // it and the image is multiplied by w_i^(m_y + n_y) at the end.  The staged
 // coefficients a[k][r] = f_{deg-r,k} q^{-C(k,2)} (top-aligned in r, zero past
 // the degree) and the window w[t] = q^{C(x0+t,2)} are signed representatives
-// (|v| < 2^30): 7 products accumulate exactly in an int64, then one fold
-// S = hi 2^32 + lo -> hi (2^32 mod p) + lo keeps |S| < 2^53.
-__device__ __forceinline__ int64_t fold64(int64_t s, uint32_t c32) { return rs_fold64(s, c32); }
+// (|v| < 2^30), so 7 products stay below 7 2^60 in magnitude.  The sums are
+// unsigned 64-bit words that start at p 2^32 (0 mod p, and above 7 2^60), so
+// they never go below zero; after every 7 rows a fold hi 2^32 + lo ->
+// hi (2^32 mod p) + lo + p 2^32 (2^32 mod p <= 2^21 for every table prime)
+// starts the next.  At the end the high word, below 2 p, loses p if it can,
+// which leaves less than p 2^32 for one REDC.
+//
+// One rolled loop over blocks of 8 columns serves every block of f and g: the
+// values go through the thread's own shared-memory column, which is read back
+// into the register array.  Fully unrolled over the register array the
+// evaluation was more code than the remainder sequence, most of it not
+// products: limits read per column, sums cleared and finished, signs and
+// selects around the shuffle (6,026 instructions per warp and chunk at
+// deg_x 24, deg_y 36, now under 4,500, of which 1,000 are products).
+// G1 with deg_x = 24, ns per image, unrolled and now (double steps in both):
+//   deg_y       14     22     28     38     44     52     60     68
+//   unrolled 0.284  0.404  0.578  0.817  1.075  1.389  1.802  2.081
+//   rolled   0.265  0.363  0.512  0.742  0.978  1.237  1.593  1.845
+// Signed sums that start at 0 (8 rows before the first fold) measured 1-3%
+// slower beyond 8 rows and 2% faster up to them.
 
-__device__ __forceinline__ uint32_t finish64(int64_t s, const ModP &m) {
-  return redc((uint64_t)(s + ((int64_t)m.p << 22)), m.p, m.pinv);  // 0 <= . < 2^54 < p 2^32
+// Rows of one parity of a polynomial of x-degree mx (both parities have the
+// same number; the last row may be a zero row), and the distance in words
+// between the two parities: 16 mod 32, so that the two lanes of a point pair
+// read different banks.
+__host__ __device__ __forceinline__ int g1_half_rows(int mx) { return (mx >> 1) + 1; }
+__host__ __device__ __forceinline__ int g1_odd_offset(int mx, int C) {
+  const int w = g1_half_rows(mx) * C;
+  return w + ((48 - (w & 31)) & 31);
 }
+__host__ __device__ __forceinline__ int g1_poly_words(int mx, int C) { return g1_odd_offset(mx, C) + g1_half_rows(mx) * C; }
 
+// Values of f_j (or g_j) at +q^i (lane par = 0) and, negated, at -q^i (lane
+// par = 1), j from the top: E + xO and xO - E from the partner lane's part.
+// The sign of the second is the same for every coefficient of f and g; the
+// image takes it back.  sa: staged coefficients of this lane's parity; steps:
+// rows per block of 8 columns; win: the window at this point pair and parity;
+// col: this thread's C words of shared memory.
 template <int C>
-__device__ __forceinline__ void eval_chirp(uint32_t (&P)[C], const int32_t *sa, const int2 *meta,
-                                           int deg, const int32_t *win, int par, const ModP &m) {
-  const uint32_t c32 = m.r1;  // 2^32 mod p (<= 2^21 for every table prime)
+__device__ __forceinline__ void eval_chirp(uint32_t (&P)[C], const int32_t *sa, const int32_t *steps,
+                                           const int32_t *win, uint32_t *col, int par, const ModP &m) {
+  const uint32_t c32 = m.r1;  // 2^32 mod p
+  const uint32_t sg = par ? 1u : 0u - 1u, off = par ? 0u : m.p;  // sent: O, or p - E
+  uint32_t *pc = col;
+#pragma unroll 1
+  for (int b = 0; b < C / 8; ++b) {
+    const int32_t *pa = sa + 8 * b;
+    const int32_t *pw = win;
+    uint64_t acc[8];
 #pragma unroll
-  for (int r0 = 0; r0 < C; r0 += 8) {
-    int64_t acc[8];
-#pragma unroll
-    for (int rr = 0; rr < 8; ++rr) acc[rr] = 0;
-    int kmax = -1;
-#pragma unroll
-    for (int rr = 0; rr < 8; ++rr)
-      if (deg - (r0 + rr) >= 0) kmax = max(kmax, meta[deg - (r0 + rr)].y);
-    auto step = [&](int k) {
-      const int32_t c = win[k];
-      const int4 lo = *reinterpret_cast<const int4 *>(sa + k * C + r0);
-      const int4 hi = *reinterpret_cast<const int4 *>(sa + k * C + r0 + 4);
-      acc[0] = rs_mac_s32(acc[0], lo.x, c);
-      acc[1] = rs_mac_s32(acc[1], lo.y, c);
-      acc[2] = rs_mac_s32(acc[2], lo.z, c);
-      acc[3] = rs_mac_s32(acc[3], lo.w, c);
-      acc[4] = rs_mac_s32(acc[4], hi.x, c);
-      acc[5] = rs_mac_s32(acc[5], hi.y, c);
-      acc[6] = rs_mac_s32(acc[6], hi.z, c);
-      acc[7] = rs_mac_s32(acc[7], hi.w, c);
+    for (int r = 0; r < 8; ++r) acc[r] = (uint64_t)m.p << 32;
+    auto step = [&](int u) {
+      const int64_t c = pw[2 * u];
+      const int4 lo = *reinterpret_cast<const int4 *>(pa + u * C);
+      const int4 hi = *reinterpret_cast<const int4 *>(pa + u * C + 4);
+      acc[0] += (uint64_t)(lo.x * c);
+      acc[1] += (uint64_t)(lo.y * c);
+      acc[2] += (uint64_t)(lo.z * c);
+      acc[3] += (uint64_t)(lo.w * c);
+      acc[4] += (uint64_t)(hi.x * c);
+      acc[5] += (uint64_t)(hi.y * c);
+      acc[6] += (uint64_t)(hi.z * c);
+      acc[7] += (uint64_t)(hi.w * c);
     };
-    // rows par, par + 2, ... (window entry k): full groups of 7 products per
-    // fold unrolled, then the rest
-    int k = par;
+    int n = steps[b];
 #pragma unroll 1
-    for (; k + 12 <= kmax; k += 14) {
+    for (; n >= 7; n -= 7) {
 #pragma unroll
-      for (int u = 0; u < 7; ++u) step(k + 2 * u);
+      for (int u = 0; u < 7; ++u) step(u);
+      pa += 7 * C;
+      pw += 14;
 #pragma unroll
-      for (int rr = 0; rr < 8; ++rr) acc[rr] = fold64(acc[rr], c32);
+      for (int r = 0; r < 8; ++r)
+        acc[r] = (acc[r] >> 32) * c32 + (((uint64_t)m.p << 32) | (uint32_t)acc[r]);
     }
-#pragma unroll 1
-    for (; k <= kmax; k += 2) step(k);
+    if (n & 4) {
 #pragma unroll
-    for (int rr = 0; rr < 8; ++rr) acc[rr] = fold64(acc[rr], c32);
+      for (int u = 0; u < 4; ++u) step(u);
+      pa += 4 * C;
+      pw += 8;
+    }
+    if (n & 2) {
 #pragma unroll
-    for (int rr = 0; rr < 8; ++rr) P[r0 + rr] = kmax >= 0 ? finish64(acc[rr], m) : 0u;
+      for (int u = 0; u < 2; ++u) step(u);
+      pa += 2 * C;
+      pw += 4;
+    }
+    if (n & 1) step(0);
+#pragma unroll
+    for (int r = 0; r < 8; ++r) {
+      const uint32_t h = (uint32_t)(acc[r] >> 32);  // < 15 2^28 + 2^21 < 2 p
+      const uint32_t v = redc(((uint64_t)rs_umin(h, h - m.p) << 32) | (uint32_t)acc[r], m.p, m.pinv);
+      const uint32_t s = v + __shfl_xor_sync(0xffffffffu, v * sg + off, 1);  // < 2 p
+      pc[r] = rs_umin(s, s - m.p);
+    }
+    pc += 8;
   }
+#pragma unroll
+  for (int r = 0; r < C; ++r) P[r] = col[r];
 }
 
-// f_j(+-x) = E_j +- x O_j from the partner lane's part: lane par = 0 holds
-// E_j and keeps +x, lane par = 1 holds x O_j and takes -x.
-template <int C>
-__device__ __forceinline__ void combine_pm(uint32_t (&P)[C], int par, const ModP &m) {
-#pragma unroll
-  for (int r = 0; r < C; ++r) {
-    const uint32_t other = __shfl_xor_sync(0xffffffffu, P[r], 1);
-    const uint32_t e = par ? other : P[r], o = par ? P[r] : other;
-    P[r] = par ? msub(e, o, m.p) : madd(e, o, m.p);
-  }
-}
-
-// a[k][r] for k <= dx (the largest x-degree), r < C; qn[t] = q^{-C(t,2)}.
+// Row k of the staged coefficients, k < 2 g1_half_rows(dx); qn[t] = q^{-C(t,2)}.
 template <int C>
 __device__ __forceinline__ void stage_chirp(int32_t *sa, const int2 *smeta, int deg, int dx,
                                             const uint32_t *limbs, int stride, int L,
                                             const uint32_t *V, const uint32_t *qn, const ModP &m) {
-  const int n = (dx + 1) * C;
+  const int n = 2 * g1_half_rows(dx) * C, odd = g1_odd_offset(dx, C);
   for (int idx = threadIdx.x; idx < n; idx += blockDim.x) {
     const int k = idx / C, r = idx - k * C, j = deg - r;
     int32_t v = 0;
     if (j >= 0 && k <= smeta[j].y)
       v = signed_rep(mmul(reduce_coef(limbs + ((size_t)k * stride + j) * L, L, V, m), qn[k], m), m.p);
-    sa[idx] = v;
+    sa[(k & 1) * odd + (k >> 1) * C + r] = v;
   }
 }
 
@@ -430,9 +466,11 @@ __global__ void __launch_bounds__(128, RS_G1_MINB) g1_kernel(G1Args a) {
     const int nmeta = pd.my + pd.ny + 2;
     const int dxm = max(pd.mxf, pd.mxg);
     int2 *smeta = reinterpret_cast<int2 *>(sm);
-    int32_t *saf = reinterpret_cast<int32_t *>(sm) + ((2 * nmeta + 7) & ~7);  // 32-byte aligned
-    int32_t *sag = saf + (pd.mxf + 1) * C;
-    int32_t *swin = sag + (pd.mxg + 1) * C;
+    int32_t *ssteps = reinterpret_cast<int32_t *>(sm) + 2 * nmeta;  // rows per parity of each block of 8 columns
+    int32_t *saf = reinterpret_cast<int32_t *>(sm) + ((2 * nmeta + 2 * (C / 8) + 7) & ~7);  // 32-byte aligned
+    int32_t *sag = saf + ((g1_poly_words(pd.mxf, C) + 7) & ~7);
+    int32_t *swin = sag + g1_poly_words(pd.mxg, C);
+    uint32_t *scol = reinterpret_cast<uint32_t *>(swin) + (blockDim.x >> 1) + dxm + 2 + threadIdx.x * (C + 1);  // odd stride
     const size_t tb = (size_t)tl.prime * a.tstride;
 
     for (int i = threadIdx.x; i < nmeta; i += blockDim.x) smeta[i] = a.meta[pd.meta_off + i];
@@ -440,12 +478,19 @@ __global__ void __launch_bounds__(128, RS_G1_MINB) g1_kernel(G1Args a) {
     stage_chirp<C>(saf, smeta, pd.my, pd.mxf, a.limbs + pd.f_off, pd.fstride, pd.Lf, V, a.qn + tb, m);
     stage_chirp<C>(sag, smeta + pd.my + 1, pd.ny, pd.mxg, a.limbs + pd.g_off, pd.gstride, pd.Lg, V,
                    a.qn + tb, m);
+    for (int i = threadIdx.x; i < 2 * (C / 8); i += blockDim.x) {
+      const int w = i / (C / 8), top = (w ? pd.ny : pd.my) - 8 * (i - w * (C / 8));
+      int k = -2;
+      for (int r = 0; r < 8; ++r)
+        if (top - r >= 0) k = max(k, smeta[w * (pd.my + 1) + top - r].y);
+      ssteps[i] = (k >> 1) + 1;  // x-degree -1 (a zero coefficient): no row
+    }
     __syncthreads();
 
     if (tl.x0 == 0 && threadIdx.x == 0) {  // unlucky prime: a leading coefficient vanishes mod p
       bool zf = true, zg = true;
-      for (int k = 0; k <= pd.mxf; ++k) zf = zf && saf[k * C] == 0;
-      for (int k = 0; k <= pd.mxg; ++k) zg = zg && sag[k * C] == 0;
+      for (int k = 0; k <= pd.mxf; ++k) zf = zf && saf[(k & 1) * g1_odd_offset(pd.mxf, C) + (k >> 1) * C] == 0;
+      for (int k = 0; k <= pd.mxg; ++k) zg = zg && sag[(k & 1) * g1_odd_offset(pd.mxg, C) + (k >> 1) * C] == 0;
       if (zf || zg) atomicAdd(a.stats + ST_UNLUCKY_PRIMES, 1ull);
     }
 
@@ -455,17 +500,15 @@ __global__ void __launch_bounds__(128, RS_G1_MINB) g1_kernel(G1Args a) {
     const int half = (int)(blockDim.x >> 1);
     for (int cx = tl.x0; cx < tl.x0 + tl.n; cx += half) {
       const int nn = min(half, tl.x0 + tl.n - cx);
-      for (int t = threadIdx.x; t < half + dxm + 1; t += blockDim.x) swin[t] = a.qc[tb + cx + t];
+      for (int t = threadIdx.x; t < half + dxm + 2; t += blockDim.x) swin[t] = a.qc[tb + cx + t];
       __syncthreads();
       uint32_t unlucky = 0u, degen = 0u;
       const int i = cx + ti;  // point pair: this thread's image is at (-1)^par q^i
       // every thread evaluates (the shuffles need the whole warp); only the
       // threads of the chunk's pairs run the remainder sequence
       uint32_t A[C], B[C];
-      eval_chirp<C>(A, saf, smeta, pd.my, swin + ti, par, m);
-      eval_chirp<C>(B, sag, smeta + pd.my + 1, pd.ny, swin + ti, par, m);
-      combine_pm<C>(A, par, m);
-      combine_pm<C>(B, par, m);
+      eval_chirp<C>(A, saf + par * g1_odd_offset(pd.mxf, C), ssteps, swin + ti + par, scol, par, m);
+      eval_chirp<C>(B, sag + par * g1_odd_offset(pd.mxg, C), ssteps + C / 8, swin + ti + par, scol, par, m);
       if (ti < nn) {
         unlucky = (A[0] == 0u || B[0] == 0u) ? 1u : 0u;
         Prs s;
@@ -473,7 +516,7 @@ __global__ void __launch_bounds__(128, RS_G1_MINB) g1_kernel(G1Args a) {
         s.b = pd.ny;
         s.num = s.den = s.Q = m.r1;
         s.eprev = max(min(pd.my, pd.ny) - 1, 0);
-        s.sign = 0u;
+        s.sign = (uint32_t)(par & (pd.my + pd.ny));  // A and B are negated in odd lanes
         s.degen = 0u;
         prs_run<C>(A, B, s, m);
         // the chirp factor left out of the coefficients (reloaded: no register held through the sequence)

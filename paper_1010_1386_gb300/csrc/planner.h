@@ -40,13 +40,21 @@ struct PairPlan {
 int rs_plan_pair(const rs_bipoly *f, const rs_bipoly *g, const std::vector<double> &log2p,
                  PairPlan &plan, const char **why);
 
-// Shared-memory words one G1 tile of `threads` points stages for plan p in
-// register-capacity class C: per-j x-degrees, chirp-scaled coefficients of
-// f and g ([x-degree + 1][C] each) and the window of q^{C(t,2)}.
+// Words of per-j x-degrees, chirp-scaled coefficients of f and g ([x-degree +
+// 1][C] each) and the window of q^{C(t,2)} for a tile of `threads` points: the
+// measure the planner's limit on staged inputs is stated in.
 inline int rs_g1_staged_words(const PairPlan &p, int C, int threads) {
   const int meta = (2 * (p.f.my + p.g.my + 2) + 7) & ~7;
   const int dx = p.f.mx > p.g.mx ? p.f.mx : p.g.mx;
   return meta + (p.f.mx + 1) * C + (p.g.mx + 1) * C + threads + dx;
+}
+
+// Shared-memory words of a G1 tile of `threads` points of plan p in
+// register-capacity class C, an upper bound: the above with the rows split by
+// parity (a row and up to 31 words more per polynomial), the row counts per
+// block of 8 columns, and one column of C + 1 words per thread.
+inline int rs_g1_smem_words(const PairPlan &p, int C, int threads) {
+  return rs_g1_staged_words(p, C, threads) + 2 * (C + 31 + 8) + 2 * (C / 8) + 8 + (C + 1) * threads;
 }
 
 // Primes in (2^31 - 2^20, 2^31), descending, by a sieve of Eratosthenes.

@@ -8,7 +8,7 @@
 
 #define RS_VT_STRIDE (RS_MAX_LIMBS + 1)  // V[k][l] = 2^(32 l) R^2 mod p_k, l = 0..RS_MAX_LIMBS
 #define RS_G1_MAX_STAGED_WORDS (48 * 1024)  // staged residues + meta per G1 tile
-#define RS_G1_MAX_SMEM_BYTES (RS_G1_MAX_STAGED_WORDS * 4)
+#define RS_G1_MAX_SMEM_BYTES (226 * 1024)  // of 227 KB, next to the kernel's static word
 #define RS_G2_PAD 8          // zero words around each G2 shared-memory region
 #define RS_CONV_R 7          // G2 outputs per register block; odd, so lanes hit distinct banks
 #define RS_G2_MAX_SMEM_BYTES (4 * (8192 + 2 * RS_G2_PAD) * 4)  // four regions of M <= 8192 pairs

@@ -1,8 +1,10 @@
-"""The remainder sequence's double steps (two degrees of one polynomial per
+"""The image kernel.  The remainder sequence's double steps (two degrees of one polynomial per
 pass): every image equals the oracle's determinant of the formal Sylvester
 matrix, over degrees at the edges of the register capacities and phases,
 equal, adjacent and far apart, on dense inputs and on sparse ones whose
-sequence meets vanishing pivots."""
+sequence meets vanishing pivots; the evaluation's row groups (7 products per
+fold, two parities) at their edges, with zero coefficients and inputs so large
+that a block takes fewer threads."""
 import random
 
 import pytest
@@ -70,3 +72,23 @@ def test_vanishing_pivots(ctx, m, n):
     if m <= 69:
         ps, xs, zs = ctx.images(times(f, h), times(g, h), 2, 6)
         assert not zs.any()
+
+
+@pytest.mark.parametrize("dx", [0, 1, 2, 5, 6, 11, 12, 13, 14, 15, 16, 26, 27, 28, 29, 41, 42, 43])
+def test_evaluation_rows(ctx, dx):
+    rng = random.Random(31 * dx + 5)
+    for m, n, other in ((9, 9, 3), (17, 3, dx), (33, 10, 1)):
+        f, g = rand_bipoly(rng, dx, m, 33), rand_bipoly(rng, other, n, 33)
+        for j in (1, m // 2):  # zero coefficients of y^j, and one of low x-degree
+            for row in f:
+                row[j] = 0
+        for row in g[1:]:
+            row[n // 2] = 0
+        check(ctx, f, g, primes=1, points=70)
+
+
+def test_largest_staged_inputs(ctx):
+    """deg_y = 71 with deg_x = 470 and 190: the staged coefficients leave too
+    little shared memory for 128 threads' columns."""
+    rng = random.Random(9)
+    check(ctx, rand_bipoly(rng, 470, 71, 12), rand_bipoly(rng, 190, 1, 12), primes=1, points=4)
