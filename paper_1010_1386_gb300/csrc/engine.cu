@@ -58,38 +58,44 @@ int rs_fail(rs_ctx *c, int code, const std::string &msg) {
 
 // ------------------------------------------------------------------ planning
 
+// Host threads for planning n pairs, and pairs per task.  Planning reads every
+// input coefficient once and takes one summed autocorrelation per polynomial
+// ((deg_x + 1)^2 (deg_y + 1) / 2 products); on the Grace host it takes about
+// 0.6 us per polynomial, 5 ns per coefficient and 1 ns per limb, and 0.5 ns
+// per product.  From 60 us on the pairs are shared: a worker takes a few
+// microseconds to wake.
+static int plan_threads(int n, const rs_bipoly *f, const rs_bipoly *g, int *step) {
+  auto cost = [](const rs_bipoly &p) {  // ns
+    if (!p.coeffs || p.deg_x < 0 || p.deg_y < 0 || p.limbs < 1 || p.limbs > RS_MAX_LIMBS) return 0.0;
+    const double c = ((double)p.deg_x + 1) * ((double)p.deg_y + 1);
+    return 600.0 + c * (5.0 + p.limbs) + (c <= 0x1p26 ? 0.25 * c * (p.deg_x + 1) : 0.0);
+  };
+  double ns = 0.0;
+  for (int i = 0; i < n; ++i) ns += cost(f[i]) + cost(g[i]);
+  const int threads = ns < 60e3 ? 1 : (int)std::min(16.0, ns / 20e3);
+  *step = std::max(1, n / (8 * threads));
+  return threads;
+}
+
+static void plan_one(rs_ctx *ctx, const rs_bipoly &f, const rs_bipoly &g, PairPlan &plan, const char **why) {
+  try {
+    plan.status = rs_plan_pair(&f, &g, ctx->log2p, plan, why);
+  } catch (const std::exception &) {
+    plan.status = RS_ERR_NOMEM;
+    *why = "out of host memory";
+  }
+}
+
 int rs_plan_all(rs_ctx *ctx, int n, const rs_bipoly *f, const rs_bipoly *g,
                 std::vector<PairPlan> &plans, int32_t *status, int *first_err) {
   plans.assign(n, PairPlan());
   *first_err = RS_OK;
   std::vector<const char *> why(n, "");
-  auto plan_range = [&](int lo, int hi) {
-    for (int i = lo; i < hi; ++i) plans[i].status = rs_plan_pair(&f[i], &g[i], ctx->log2p, plans[i], &why[i]);
-  };
-  // Planning reads every input coefficient once and takes one summed
-  // autocorrelation per polynomial ((deg_x + 1)^2 (deg_y + 1) / 2 products);
-  // large batches are split over host threads in contiguous ranges of pairs.
-  auto sane = [](const rs_bipoly &p) {
-    return p.coeffs && p.deg_x >= 0 && p.deg_y >= 0 && p.deg_x < (1 << 26) && p.deg_y < (1 << 26) &&
-           p.limbs >= 1 && p.limbs <= RS_MAX_LIMBS;
-  };
-  int64_t words = 0;  // only steers the thread count
-  auto corr = [](const rs_bipoly &p) {  // sane p: (deg_x + 1)^2 (deg_y + 1) < 2^78 would overflow
-    const int64_t c = (int64_t)(p.deg_x + 1) * (p.deg_y + 1);
-    return c <= ((int64_t)1 << 26) ? c * (p.deg_x + 1) / 16 : 0;
-  };
-  for (int i = 0; i < n; ++i)
-    if (sane(f[i]) && sane(g[i])) words += rs_input_words(f[i]) + rs_input_words(g[i]) + corr(f[i]) + corr(g[i]);
-  const int hw = std::max(1, (int)std::thread::hardware_concurrency());
-  const int nt = (int)std::min<int64_t>({(int64_t)std::min(hw, 16), (int64_t)n, words / (int64_t(1) << 18) + 1});
-  if (nt <= 1) {
-    plan_range(0, n);
-  } else {
-    std::vector<std::thread> th;
-    for (int t = 0; t < nt; ++t)
-      th.emplace_back(plan_range, (int)((int64_t)n * t / nt), (int)((int64_t)n * (t + 1) / nt));
-    for (auto &x : th) x.join();
-  }
+  int step = 1;
+  const int threads = plan_threads(n, f, g, &step);
+  ctx->pool.run((n + step - 1) / step, threads, [&](int t) {
+    for (int i = t * step; i < std::min(n, (t + 1) * step); ++i) plan_one(ctx, f[i], g[i], plans[i], &why[i]);
+  });
   for (int i = 0; i < n; ++i) {
     const int rc = plans[i].status;
     if (status) status[i] = rc;
@@ -400,6 +406,7 @@ void rs_free_batch(rs_batch *b) {
     if (e) cudaEventDestroy(e);
   for (auto &e : b->jev)
     if (e) cudaEventDestroy(e);
+  for (auto &e : b->cev) cudaEventDestroy(e);
   if (b->arena) {
     if (b->opt.stream_ordered)
       cudaFreeAsync(b->arena, b->stream);
@@ -1112,10 +1119,15 @@ int rs_build_batch(rs_ctx *ctx, int n, const rs_bipoly *f, const rs_bipoly *g,
 
 int rs_upload(rs_batch *b, const rs_bipoly *f, const rs_bipoly *g) {
   rs_ctx *ctx = b->ctx;
-  for (int i = 0; i < b->n; ++i) {
-    memcpy(b->h_in + b->in_f[i], f[i].coeffs, rs_input_words(f[i]) * 4);
-    memcpy(b->h_in + b->in_g[i], g[i].coeffs, rs_input_words(g[i]) * 4);
-  }
+  // one thread copies about 10 GB/s: shared from 256 KiB on
+  const int threads = (int)std::min<int64_t>(16, b->in_words >> 15);
+  const int step = std::max(1, b->n / 64);
+  ctx->pool.run((b->n + step - 1) / step, threads, [&](int t) {
+    for (int i = t * step; i < std::min(b->n, (t + 1) * step); ++i) {
+      memcpy(b->h_in + b->in_f[i], f[i].coeffs, rs_input_words(f[i]) * 4);
+      memcpy(b->h_in + b->in_g[i], g[i].coeffs, rs_input_words(g[i]) * 4);
+    }
+  });
   if (b->in_words)
     RS_CUDA(ctx, cudaMemcpyAsync(b->d_in, b->h_in, b->in_words * 4, cudaMemcpyHostToDevice, b->stream));
   return RS_OK;
@@ -1470,61 +1482,117 @@ int rs_unpack_one(rs_batch *b, int i, std::vector<uint32_t> &words, int *deg, in
   if (p.status != RS_OK) return p.status;
   if (device_status(b) != RS_OK) return RS_ERR_TIMEOUT;
   const uint32_t *w = result_shape(b, i, deg, limbs);
-  words.assign((size_t)(*deg + 1) * *limbs, 0u);
-  for (int j = 0; j <= *deg; ++j)
-    memcpy(&words[(size_t)j * *limbs], w + (size_t)j * p.Lout, (size_t)*limbs * 4);
+  try {
+    words.clear();
+    words.reserve((size_t)(*deg + 1) * *limbs);
+    for (int j = 0; j <= *deg; ++j) words.insert(words.end(), w + (size_t)j * p.Lout, w + (size_t)j * p.Lout + *limbs);
+  } catch (const std::exception &) {
+    return RS_ERR_NOMEM;
+  }
   return RS_OK;
 }
 
-static int unpack_pair(rs_batch *b, int i, rs_upoly &o) {
+// Shape of pair i's result into o, and whether its limbs can be copied there.
+static int shape_pair(rs_batch *b, int i, rs_upoly &o) {
   const PairPlan &p = b->plans[i];
   int rc = p.status;
   if (rc == RS_OK && !o.coeffs && o.capacity_words > 0) rc = RS_ERR_ARG;
   if (rc != RS_OK) return rc;
   int deg, L;
-  const uint32_t *w = result_shape(b, i, &deg, &L);
+  result_shape(b, i, &deg, &L);
   o.deg = deg;
   o.limbs = L;
-  if ((int64_t)(deg + 1) * L > o.capacity_words) return RS_ERR_CAPACITY;
-  if (L == p.Lout) {
-    if (deg >= 0) memcpy(o.coeffs, w, (size_t)(deg + 1) * L * 4);
-  } else {
-    for (int j = 0; j <= deg; ++j) memcpy(o.coeffs + (size_t)j * L, w + (size_t)j * p.Lout, (size_t)L * 4);
-  }
-  return RS_OK;
+  return (int64_t)(deg + 1) * L > o.capacity_words ? RS_ERR_CAPACITY : RS_OK;
 }
 
-int rs_unpack(rs_batch *b, rs_upoly *out, int32_t *status) {
+// Results to the caller's buffers: the shapes (and the status word) are copied
+// back first, then the limbs in pieces; while one piece is on its way the host
+// threads trim and copy the one before out of the staging buffer.
+static int fetch(rs_batch *b, rs_upoly *out, int32_t *status) {
   rs_ctx *ctx = b->ctx;
+  DevGuard dg(ctx->device);
+  if (!b->ran) return rs_fail(ctx, RS_ERR_STATE, "batch has not been run");
   const int n = b->n;
-  if (device_status(b) != RS_OK) {
-    for (int i = 0; i < n && status; ++i) status[i] = RS_ERR_TIMEOUT;
-    return rs_fail(ctx, RS_ERR_TIMEOUT, "tensor-core kernels: a bounded device wait ran out");
+  const int64_t limbs_words = std::min(b->shape_off, b->out_words);
+  // Pieces of at least 16 MiB (the copy runs at about 190 GB/s, and each piece
+  // wakes the host threads once), cut between pairs.
+  const int64_t piece = std::max<int64_t>((int64_t)1 << 22, limbs_words / 8 + 1);
+  std::vector<int64_t> ends;  // word offsets
+  std::vector<int> pair_end;  // pairs complete at each end
+  for (int i = 0; i < n; ++i) {
+    const int d = b->dev_index[i];
+    if (d < 0) continue;
+    const int64_t e = b->descs[d].out_off + (int64_t)b->plans[i].N * b->plans[i].Lout;
+    if (e - (ends.empty() ? 0 : ends.back()) >= piece) {
+      ends.push_back(e);
+      pair_end.push_back(i + 1);
+    }
+  }
+  if (ends.empty() || ends.back() < limbs_words) {
+    ends.push_back(limbs_words);
+    pair_end.push_back(n);
+  }
+  pair_end.back() = n;
+  const int np = (int)ends.size();
+  while (np > 1 && (int)b->cev.size() < np) {
+    cudaEvent_t ev = nullptr;
+    RS_CUDA(ctx, cudaEventCreateWithFlags(&ev, cudaEventDisableTiming));
+    b->cev.push_back(ev);
+  }
+  cudaError_t e = cudaSuccess;
+  if (np == 1 && b->out_words)  // small results: everything in one copy
+    e = cudaMemcpyAsync(b->h_out, b->d_out, b->out_words * 4, cudaMemcpyDeviceToHost, b->stream);
+  if (np > 1 && b->out_words > limbs_words)
+    e = cudaMemcpyAsync(b->h_out + limbs_words, b->d_out + limbs_words, (b->out_words - limbs_words) * 4,
+                        cudaMemcpyDeviceToHost, b->stream);
+  for (int c = 0; c < np && np > 1 && e == cudaSuccess; ++c) {
+    const int64_t at = c ? ends[c - 1] : 0;
+    if (ends[c] > at)
+      e = cudaMemcpyAsync(b->h_out + at, b->d_out + at, (ends[c] - at) * 4, cudaMemcpyDeviceToHost, b->stream);
+    if (e == cudaSuccess) e = cudaEventRecord(b->cev[c], b->stream);
   }
   std::vector<int> rcs(n, RS_OK);
-  // Large outputs are trimmed and copied by several host threads, each
-  // taking a contiguous range of pairs of about equal size.
-  const int64_t kWordsPerThread = int64_t(1) << 20;
-  const int hw = std::max(1, (int)std::thread::hardware_concurrency());
-  const int nt = (int)std::min<int64_t>({(int64_t)std::min(hw, 16), (int64_t)n, b->out_words / kWordsPerThread + 1});
-  if (nt <= 1) {
-    for (int i = 0; i < n; ++i) rcs[i] = unpack_pair(b, i, out[i]);
-  } else {
-    std::vector<int> cut(1, 0);
-    int64_t acc = 0;
-    for (int i = 0; i < n; ++i) {
-      const PairPlan &p = b->plans[i];
-      if (p.status == RS_OK && !p.trivial_zero) acc += (int64_t)p.N * p.Lout;
-      if (acc * nt >= b->out_words * (int64_t)cut.size() && (int)cut.size() < nt) cut.push_back(i + 1);
+  struct Rows {  // rows [j0, j1) of pair i
+    int i, j0, j1;
+  };
+  std::vector<Rows> rows;
+  for (int c = 0; c < np && e == cudaSuccess; ++c) {
+    e = np > 1 ? cudaEventSynchronize(b->cev[c]) : cudaStreamSynchronize(b->stream);
+    if (e != cudaSuccess) break;
+    if (c == 0 && device_status(b) != RS_OK) {
+      cudaStreamSynchronize(b->stream);  // the other pieces still arrive in the staging buffer
+      for (int i = 0; i < n && status; ++i) status[i] = RS_ERR_TIMEOUT;
+      return rs_fail(ctx, RS_ERR_TIMEOUT, "tensor-core kernels: a bounded device wait ran out");
     }
-    while ((int)cut.size() <= nt) cut.push_back(n);
-    cut.back() = n;
-    std::vector<std::thread> th;
-    for (int t = 0; t < nt; ++t)
-      th.emplace_back([&, t] {
-        for (int i = cut[t]; i < cut[t + 1]; ++i) rcs[i] = unpack_pair(b, i, out[i]);
-      });
-    for (auto &x : th) x.join();
+    rows.clear();
+    int64_t words = 0;
+    for (int i = c ? pair_end[c - 1] : 0; i < pair_end[c]; ++i) {
+      rcs[i] = shape_pair(b, i, out[i]);
+      if (rcs[i] != RS_OK || out[i].deg < 0) continue;
+      const int R = out[i].deg + 1, L = out[i].limbs;
+      const int per = std::max(1, (1 << 16) / L);  // 256 KiB a task
+      for (int j = 0; j < R; j += per) rows.push_back(Rows{i, j, std::min(R, j + per)});
+      words += (int64_t)R * L;
+    }
+    // a task of a few small pairs, or of one run of rows; a thread per 128 KiB
+    const int step = std::max<int>(1, (int)(rows.size() / 64));
+    ctx->pool.run(((int)rows.size() + step - 1) / step, (int)std::min<int64_t>(16, words >> 15), [&](int t) {
+      for (int k = t * step; k < std::min((int)rows.size(), (t + 1) * step); ++k) {
+        const Rows &r = rows[k];
+        const rs_upoly &o = out[r.i];
+        const int Lout = b->plans[r.i].Lout, L = o.limbs;
+        const uint32_t *w = b->h_out + b->descs[b->dev_index[r.i]].out_off;
+        if (L == Lout) {
+          memcpy(o.coeffs + (size_t)r.j0 * L, w + (size_t)r.j0 * L, (size_t)(r.j1 - r.j0) * L * 4);
+        } else {
+          for (int j = r.j0; j < r.j1; ++j) memcpy(o.coeffs + (size_t)j * L, w + (size_t)j * Lout, (size_t)L * 4);
+        }
+      }
+    });
+  }
+  if (e != cudaSuccess) {
+    cudaStreamSynchronize(b->stream);
+    return rs_fail(ctx, rs_cuda_code(e), std::string("result copy: ") + cudaGetErrorString(e));
   }
   int first = RS_OK;
   for (int i = 0; i < n; ++i) {
@@ -1536,15 +1604,6 @@ int rs_unpack(rs_batch *b, rs_upoly *out, int32_t *status) {
     }
   }
   return first;
-}
-
-static int fetch(rs_batch *b, rs_upoly *out, int32_t *status) {
-  rs_ctx *ctx = b->ctx;
-  DevGuard dg(ctx->device);
-  int rc = rs_fetch_async(b);
-  if (rc != RS_OK) return rc;
-  RS_CUDA(ctx, cudaStreamSynchronize(b->stream));
-  return rs_unpack(b, out, status);
 }
 
 static RsBatchOpts default_opts(rs_ctx *ctx) {
@@ -1755,11 +1814,20 @@ int rs_batch_create(rs_ctx *ctx, int32_t n, const rs_bipoly *f, const rs_bipoly 
 
 int rs_batch_upload(rs_batch *b, int32_t n, const rs_bipoly *f, const rs_bipoly *g) {
   if (!b || n != b->n || (n > 0 && (!f || !g))) return rs_fail(b ? b->ctx : nullptr, RS_ERR_ARG, "bad arguments");
-  std::vector<PairPlan> plans;
-  int first = RS_OK;
-  rs_plan_all(b->ctx, n, f, g, plans, nullptr, &first);
+  // Each pair is planned and compared by one task, which frees the plan again.
+  std::vector<char> same(n, 0);
+  int step = 1;
+  const int threads = plan_threads(n, f, g, &step);
+  b->ctx->pool.run((n + step - 1) / step, threads, [&](int t) {
+    for (int i = t * step; i < std::min(n, (t + 1) * step); ++i) {
+      PairPlan plan;
+      const char *why = "";
+      plan_one(b->ctx, f[i], g[i], plan, &why);
+      same[i] = rs_same_shape(plan, b->plans[i]);
+    }
+  });
   for (int i = 0; i < n; ++i)
-    if (!rs_same_shape(plans[i], b->plans[i]))
+    if (!same[i])
       return rs_fail(b->ctx, RS_ERR_STATE, "inputs do not match the batch's plan (pair " + std::to_string(i) + ")");
   DevGuard dg(b->ctx->device);
   return rs_upload(b, f, g);

@@ -8,6 +8,7 @@
 #include <string>
 #include <vector>
 
+#include "hostpool.h"
 #include "planner.h"
 #include "rs_internal.cuh"
 
@@ -66,6 +67,7 @@ struct rs_ctx {
   RsTables tab;
   std::vector<RsTables> retired;
   RsServer *server = nullptr;
+  RsHostPool pool;  // host threads for planning and copying results out
   std::mutex prep_mu;  // kernel attributes and the occupancy cache below
   bool g2_ready = false;
   std::map<int64_t, int> g1_occupancy;  // (capacity, threads, staged KiB) -> blocks per SM
@@ -203,6 +205,7 @@ struct rs_batch {
   cudaEvent_t ev[5] = {nullptr, nullptr, nullptr, nullptr, nullptr};  // stage bounds; [4] before Yun
   cudaEvent_t fev[2] = {nullptr, nullptr};  // fork points of the G1 and G2 stages
   std::vector<cudaEvent_t> jev;             // joins of the branches (one per launch of a forked stage)
+  std::vector<cudaEvent_t> cev;             // ends of the pieces of a large result copy
   bool ran = false;
   rs_batch_info info;
 };
@@ -234,7 +237,6 @@ void rs_batch_sizes(const std::vector<PairPlan> &plans, const rs_bipoly *f, cons
 int rs_upload(rs_batch *b, const rs_bipoly *f, const rs_bipoly *g);
 int rs_run(rs_batch *b);
 int rs_fetch_async(rs_batch *b);                                // enqueue the result copy
-int rs_unpack(rs_batch *b, rs_upoly *out, int32_t *status);     // after the copy completed
 // Unpack pair i into a freshly sized host vector (deg, limbs); returns status.
 int rs_unpack_one(rs_batch *b, int i, std::vector<uint32_t> &words, int *deg, int *limbs);
 void rs_free_batch(rs_batch *b);

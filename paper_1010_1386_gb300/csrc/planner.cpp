@@ -165,7 +165,7 @@ int analyze(const rs_bipoly *f, PolyInfo &pi, const char **why) {
   std::vector<int> dx(ny, -1);
   // ||f_j||_1 per row j, kept as sums of hi by limb position (hi < 2^64 + 1,
   // at most 2^26 terms: the sums stay far below the double range).
-  std::vector<double> acc((size_t)ny * (RS_MAX_LIMBS + 1), 0.0);
+  std::vector<double> acc((size_t)ny * L, 0.0);
   std::vector<int> tmax(ny, -1);
   int maxbits = 0;  // |c| <= 2^maxbits for every coefficient
   for (int i = 0; i < nx; ++i)
@@ -181,7 +181,7 @@ int analyze(const rs_bipoly *f, PolyInfo &pi, const char **why) {
       pi.mx = std::max(pi.mx, i);
       pi.tdeg = std::max(pi.tdeg, i + j);
       pi.my = std::max(pi.my, j);
-      acc[(size_t)j * (RS_MAX_LIMBS + 1) + t] += hi;
+      acc[(size_t)j * L + t] += hi;
       tmax[j] = std::max(tmax[j], t);
     }
   pi.zero = pi.my < 0;
@@ -193,7 +193,7 @@ int analyze(const rs_bipoly *f, PolyInfo &pi, const char **why) {
   std::vector<double> rows;
   for (int j = 0; j <= pi.my; ++j) {
     pi.nc += pi.dx[j] + 1;
-    if (tmax[j] >= 0) rows.push_back(2.0 * log2_scaled_sum(&acc[(size_t)j * (RS_MAX_LIMBS + 1)], tmax[j], rel));
+    if (tmax[j] >= 0) rows.push_back(2.0 * log2_scaled_sum(&acc[(size_t)j * L], tmax[j], rel));
   }
   pi.log2_rownorm2 = std::min(lse2(rows), log2_autocorr_bound(f, pi.dx, maxbits));
   return RS_OK;

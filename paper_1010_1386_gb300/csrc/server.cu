@@ -109,11 +109,14 @@ void reap(RsServer *s) {
       ++i;
       continue;
     }
+    // results out of the staging buffer, over the context's host threads
+    s->ctx->pool.run((int)fl.reqs.size(), (int)std::min<int64_t>(16, fl.batch->out_words >> 15), [&](int r) {
+      Request *req = fl.reqs[r];
+      req->status = q == cudaSuccess ? rs_unpack_one(fl.batch, r, req->words, &req->deg, &req->limbs) : RS_ERR_CUDA;
+    });
     const auto now = Clock::now();
     for (size_t r = 0; r < fl.reqs.size(); ++r) {
       Request *req = fl.reqs[r];
-      req->status = q == cudaSuccess ? rs_unpack_one(fl.batch, (int)r, req->words, &req->deg, &req->limbs)
-                                     : RS_ERR_CUDA;
       req->state = REQ_DONE;
       req->t_done = now;
       log_request(s, req);
