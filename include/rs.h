@@ -108,14 +108,14 @@ typedef struct {
   const char *autotune_cache;  /* tuner cache file merged at rs_create (a missing file is not an
                                   error) and rewritten at rs_destroy; NULL = none.  The string
                                   is copied. */
-  int32_t crt_form;          /* Chinese remaindering digits: 0 = by the batch's shape (one thread
-                                per coefficient when there are at least 1024 coefficients per SM;
-                                else the tensor cores when some pair has at least 128 primes and
-                                the batch has 128-coefficient tiles for half the SMs, or some pair
-                                has at least 1024 primes; else tiles on the CUDA cores), 1 = CUDA
-                                cores only, 2 = tensor cores whenever the batch does not take one
-                                thread per coefficient.  With tensor-core digits the limbs
-                                sum_k v_k P_k are a tensor-core product too. */
+  int32_t crt_form;          /* Chinese remaindering: 0 = by the batch's shape (digits with one
+                                thread per coefficient when there are at least 1024 coefficients
+                                per SM, fewer with few primes; else in tiles of coefficients on the
+                                CUDA cores or on the tensor cores, by an estimate of both; the
+                                limbs sum_k v_k P_k on the tensor cores when some pair has at least
+                                24 primes and the digits come in tiles), 1 = CUDA cores only,
+                                2 = digits and limbs on the tensor cores whenever the batch does
+                                not take one thread per coefficient */
   int32_t reserved;          /* 0 */
 } rs_config;
 

@@ -120,7 +120,7 @@ int64_t rs_input_words(const rs_bipoly &p) { return (int64_t)(p.deg_x + 1) * (p.
 // ------------------------------------------------------------------ tables
 
 static void free_tables(RsTables &t) {
-  void *p[] = {t.finv, t.gtab, t.qn, t.btab, t.qc, t.qp, t.hq, t.wtab, t.p16, t.poff, t.nh};
+  void *p[] = {t.finv, t.gtab, t.qn, t.btab, t.qc, t.qp, t.hq, t.wtab, t.wtri, t.p16, t.poff, t.nh};
   for (void *x : p)
     if (x) cudaFree(x);
   t = RsTables();
@@ -347,6 +347,7 @@ int rs_ensure_tables(rs_ctx *ctx, int K, int N, int dx) {
   std::vector<int32_t> poff(nt.K + 2, 0);
   for (int k = 0; k <= nt.K; ++k) poff[k + 1] = poff[k] + p16_row(k);
   if (e == cudaSuccess) e = cudaMalloc(&nt.wtab, std::max<size_t>(1, (size_t)nt.K * (nt.K - 1) / 2) * 4);
+  if (e == cudaSuccess) e = cudaMalloc(&nt.wtri, (size_t)crt_tri_words(nt.K) * 4);
   if (e == cudaSuccess) e = cudaMalloc(&nt.p16, (size_t)poff[nt.K + 1] * 2);
   if (e == cudaSuccess) e = cudaMalloc(&nt.poff, (size_t)(nt.K + 2) * 4);
   if (e == cudaSuccess) e = cudaMalloc(&nt.nh, (size_t)(nt.K + 1) * 4);
@@ -382,7 +383,7 @@ int rs_ensure_tables(rs_ctx *ctx, int K, int N, int dx) {
     e = cudaMemcpyAsync(nt.poff, poff.data(), poff.size() * 4, cudaMemcpyHostToDevice, ctx->stream);
   if (e == cudaSuccess) e = cudaMemcpyAsync(nt.p16, p16.data(), p16.size() * 2, cudaMemcpyHostToDevice, ctx->stream);
   if (e == cudaSuccess) e = cudaMemcpyAsync(nt.nh, nh.data(), nh.size() * 4, cudaMemcpyHostToDevice, ctx->stream);
-  if (e == cudaSuccess) e = launch_crt_tables(ctx->d_mods, nt.K, nt.wtab, ctx->stream);
+  if (e == cudaSuccess) e = launch_crt_tables(ctx->d_mods, ctx->d_crt, nt.K, nt.wtab, nt.wtri, ctx->stream);
   if (e == cudaSuccess) e = cudaStreamSynchronize(ctx->stream);
   if (e != cudaSuccess) {
     free_tables(nt);
@@ -829,27 +830,58 @@ int rs_build_batch(rs_ctx *ctx, int n, const rs_bipoly *f, const rs_bipoly *g,
   // fewer than two per SM (few coefficients with many primes each).
   std::vector<int2> g3d;
   std::vector<int4> g3b;  // CRT limb chunks: 128 coefficients x one chunk per block
-  // With enough coefficients for one thread each to fill the GPU, the digits
-  // take one thread per coefficient (no warp waits on a serial triangle);
-  // otherwise the tiled kernel spreads each coefficient's work over a block.
+  // Digits: one thread per coefficient when there are enough of them for one
+  // each to fill the GPU, the fewer the primes (a thread walks its K^2 / 2
+  // products alone): from 96 per SM, 8 K per SM, 1024 per SM for any K.
+  // Otherwise tiles of 32 or 16 coefficients on the CUDA cores, or the tensor
+  // cores in tiles of 128, whichever these times (ms, fitted to the
+  // measurements below; 608 schedulers' products against one tile's chain of
+  // digit blocks per wave) say.  Limbs: on the tensor cores unless the digits
+  // took one thread per coefficient or no pair has 24 primes.
+  // CRT stage, us: CUDA-core tiles with CUDA-core limbs, with tensor-core
+  // limbs, tensor-core digits and limbs, one thread per coefficient (with the
+  // digits' earlier kernel, which took one warp through each digit block's 64
+  // steps, the first column was 79, 727, 694, 1,650 and 5,910 us in rows 3, 6,
+  // 8, 10 and 11):
+  //   coefficients  primes (avg)  tiles  + limbs  tensor  per thread
+  //     1,160         27             24      22      43      41
+  //     3,178          8             24      24      43      30
+  //       901         69             46      32      81
+  //    18,553         66            132     100     153     360
+  //     9,220        310            296     194     247
+  //     4,520        514            429     253     383
+  //     3,362        436            274     173     297
+  //     4,097        546            396     252     403
+  //    13,448        436            690     434     368
+  //     1,640      1,199            972     542     931
+  //     4,520      2,000          4,274   2,223   2,124
+  //    16,388        547          1,236     783     500
+  //    63,008        526          4,029   2,430   1,784
+  //    18,254          7             28      36              22
+  //    51,094          9             51      96     239      34
+  //    50,782         22             59      76              47
+  //    24,994         32             49      53              55
+  //   116,878         32            134     170              92
   {
-    int64_t nt32 = 0, ncoef = 0;
+    int64_t nt32 = 0, nt128 = 0, ncoef = 0;
+    int kc = 0;  // largest prime count of the Chinese remaindering
+    double nk2 = 0.0;
     for (int i : order) {
+      const int K = b->descs[b->dev_index[i]].K;
       nt32 += (b->plans[i].N + 31) / 32;
+      nt128 += (b->plans[i].N + 127) / 128;
       ncoef += b->plans[i].N;
+      kc = std::max(kc, K);
+      nk2 += (double)b->plans[i].N * K * K;
     }
-    b->g3_jt = nt32 < 2 * (int64_t)ctx->sms ? 16 : 32;
-    b->g3_perthread = ncoef >= (int64_t)RS_G3P_MIN_COEF_PER_SM * ctx->sms;
-    // Otherwise the digits go to the tensor cores when a pair has enough
-    // primes for the per-block products to matter (two 64-prime blocks) and
-    // the 128-coefficient tiles fill half the SMs, or a pair has so many
-    // primes that the products dominate; with few tiles and a few hundred
-    // primes the CUDA-core tiles of 16 coefficients spread the work wider.
-    int64_t nt128 = 0;
-    for (int i : order) nt128 += (b->plans[i].N + 127) / 128;
-    b->g3_tensor = !b->g3_perthread && !images_only && ctx->cfg.crt_form != 1 &&
-                   (ctx->cfg.crt_form == 2 ||
-                    (maxK >= RS_G3M_MIN_K && (2 * nt128 >= ctx->sms || maxK >= RS_G3M_WIDE_K)));
+    const int64_t sms = ctx->sms;
+    b->g3_jt = nt32 < 2 * sms ? 16 : 32;
+    b->g3_perthread = ncoef >= sms * std::min<int64_t>(RS_G3P_MIN_COEF_PER_SM, std::max(96, 8 * kc));
+    const double ms_tiles = std::max(1.1e-10 * nk2 * 152 / sms, 2.7e-7 * kc * kc);
+    const double ms_tensor = (double)((nt128 + sms - 1) / sms) * kc * 0.55e-3 * (1.0 + kc / 2500.0);
+    const bool tc = !b->g3_perthread && !images_only && ctx->cfg.crt_form != 1;
+    b->g3_tensor = tc && (ctx->cfg.crt_form == 2 || (kc >= RS_G3M_MIN_K && ms_tensor < ms_tiles));
+    b->g3_tlimbs = tc && (b->g3_tensor || kc >= RS_G3L_MIN_K);
   }
   for (int i : order) {
     const PairPlan &p = b->plans[i];
@@ -874,8 +906,9 @@ int rs_build_batch(rs_ctx *ctx, int n, const rs_bipoly *f, const rs_bipoly *g,
   // operand digit rows, one 64 KB chunk per 64 of the pair's primes.
   std::vector<int64_t> g3m_xoff;
   b->g3m_x_elems = 0;
-  if (b->g3_tensor) {
+  if (b->g3_tlimbs) {
     for (const int2 &t : g3) {
+      if (t.y == 0) b->descs[t.x].xd_off = b->g3m_x_elems;
       g3m_xoff.push_back(b->g3m_x_elems);
       b->g3m_x_elems += g3m_tile_elems(b->descs[t.x].K);
     }
@@ -902,8 +935,8 @@ int rs_build_batch(rs_ctx *ctx, int n, const rs_bipoly *f, const rs_bipoly *g,
     if (bhatK[lg]) rc = rs_ensure_bhat(ctx, lg, bhatK[lg]);
   if (rc == RS_OK && g2t_kmax > 0) rc = rs_ensure_g2t_btile(ctx, g2t_kmax, g2t_tiles);
   if (rc == RS_OK && b->g3_tensor) rc = rs_ensure_g3m_wtiles(ctx, (maxK + 63) / 64);
-  if (rc == RS_OK && b->g3_tensor) rc = rs_ensure_g3l_tiles(ctx, (maxK + 63) / 64);
-  if (rc == RS_OK && b->g3_tensor) {
+  if (rc == RS_OK && b->g3_tlimbs) rc = rs_ensure_g3l_tiles(ctx, (maxK + 63) / 64);
+  if (rc == RS_OK && b->g3_tlimbs) {
     // The limbs then come from the tensor cores too: one task per (digit
     // task, unit of 64 limbs) instead of the limb chunks, with the chunks
     // from the first whose prefix products reach the unit; the longest first.
@@ -1063,7 +1096,7 @@ int rs_build_batch(rs_ctx *ctx, int n, const rs_bipoly *f, const rs_bipoly *g,
       if (e2 != cudaSuccess) rc = rs_fail(ctx, RS_ERR_CUDA, std::string("G3 set-up: ") + cudaGetErrorString(e2));
       ctx->g3m_ready = e2 == cudaSuccess;
     }
-    if (rc == RS_OK && b->g3_tensor && !ctx->g3l_ready) {
+    if (rc == RS_OK && b->g3_tlimbs && !ctx->g3l_ready) {
       cudaError_t e2 = g3l_prepare();
       if (e2 != cudaSuccess) rc = rs_fail(ctx, RS_ERR_CUDA, std::string("G3 set-up: ") + cudaGetErrorString(e2));
       ctx->g3l_ready = e2 == cudaSuccess;
@@ -1171,7 +1204,7 @@ static int enqueue(rs_batch *b, bool capturing) {
   }
   RS_CUDA(ctx, cudaMemsetAsync(b->d_counters, 0, 16 * sizeof(int32_t), s));
   RS_CUDA(ctx, cudaMemsetAsync(b->d_stats, 0, ST_COUNT * sizeof(unsigned long long), s));
-  if (b->g2t_x_elems > 0 || b->g3_tensor)  // the status word only the tensor-core kernels write
+  if (b->g2t_x_elems > 0 || b->g3_tlimbs)  // the status word only the tensor-core kernels write
     RS_CUDA(ctx, cudaMemsetAsync(b->d_out + b->status_off, 0, sizeof(uint32_t), s));
   if (timing) RS_CUDA(ctx, record(b->ev[0], s, capturing));
   if (b->schur) {  // Schur variant of G1 over every tile, then the elimination fallback
@@ -1363,6 +1396,7 @@ static int enqueue(rs_batch *b, bool capturing) {
     a3.mods = ctx->d_mods;
     a3.crt = ctx->d_crt;
     a3.wtab = tab.wtab;
+    a3.wtri = tab.wtri;
     a3.p16 = tab.p16;
     a3.poff = tab.poff;
     a3.nh = tab.nh;
@@ -1373,7 +1407,8 @@ static int enqueue(rs_batch *b, bool capturing) {
     a3.shape = reinterpret_cast<int32_t *>(b->d_out + b->shape_off);
     RS_CUDA(ctx, cudaMemsetAsync(a3.shape, 0, b->descs.size() * 2 * sizeof(int32_t), s));
     a3.kmax = b->kmax;
-    a3.signed_digits = b->g3_tensor ? 1 : 0;
+    a3.signed_digits = b->g3_tlimbs ? 1 : 0;
+    a3.xdig = b->g3_tlimbs ? b->d_g3m_x : nullptr;
     if (b->g3_perthread) {
       RS_CUDA(ctx, launch_g3p(b->ng3, a3, b->d_g3, s));
     } else if (b->g3_tensor) {
@@ -1394,6 +1429,10 @@ static int enqueue(rs_batch *b, bool capturing) {
       am.err = reinterpret_cast<int32_t *>(b->d_out + b->status_off);
       am.stall = ctx->d_stall;
       RS_CUDA(ctx, launch_g3m(b->ng3, am, s));
+    } else {
+      RS_CUDA(ctx, launch_g3t(b->ng3d, a3, b->d_g3d, s, b->g3_jt));
+    }
+    if (b->g3_tlimbs) {
       G3lArgs al;
       al.pairs = b->d_pairs;
       al.tasks = b->d_g3;
@@ -1407,14 +1446,12 @@ static int enqueue(rs_batch *b, bool capturing) {
       }
       al.xl = b->d_xl;
       al.carry = b->d_cy;
-      al.err = am.err;
+      al.err = reinterpret_cast<int32_t *>(b->d_out + b->status_off);
       al.stall = ctx->d_stall;
       RS_CUDA(ctx, launch_g3l(b->ng3b, al, s));
-    } else {
-      RS_CUDA(ctx, launch_g3t(b->ng3d, a3, b->d_g3d, s, b->g3_jt));
     }
     // the output kernel; the limb chunks unless the tensor cores formed the limbs
-    RS_CUDA(ctx, launch_g3bc(b->g3_tensor ? 0 : b->ng3b, b->ng3, a3, b->d_g3, s));
+    RS_CUDA(ctx, launch_g3bc(b->g3_tlimbs ? 0 : b->ng3b, b->ng3, a3, b->d_g3, s));
   }
   if (timing) RS_CUDA(ctx, record(b->ev[3], s, capturing));
   return RS_OK;
@@ -1473,7 +1510,7 @@ static const uint32_t *result_shape(rs_batch *b, int i, int *deg, int *limbs) {
 // The device status word copied back with the results: non-zero when a
 // bounded wait of the tensor-core interpolation ran out in the last run.
 static int device_status(rs_batch *b) {
-  if ((b->g2t_x_elems == 0 && !b->g3_tensor) || b->out_words <= b->status_off || !b->h_out) return RS_OK;
+  if ((b->g2t_x_elems == 0 && !b->g3_tlimbs) || b->out_words <= b->status_off || !b->h_out) return RS_OK;
   return b->h_out[b->status_off] ? RS_ERR_TIMEOUT : RS_OK;
 }
 

@@ -37,6 +37,7 @@ struct RsTables {
   int32_t *btab = nullptr, *qc = nullptr;
   // Chinese-remaindering tables for the first K primes.
   int32_t *wtab = nullptr;   // triangular p_0 ... p_{l-1} mod p_k
+  int32_t *wtri = nullptr;   // its diagonal blocks with Garner's constants folded in
   uint16_t *p16 = nullptr;   // prefix products in 16-bit digits
   int32_t *poff = nullptr;   // K + 1 row offsets into p16
   int32_t *nh = nullptr;     // digits per prefix product
@@ -171,6 +172,7 @@ struct rs_batch {
   int g3_jt = 32;                    // coefficients per CRT digit tile (32 or 16)
   bool g3_perthread = false;         // CRT digits with one thread per coefficient
   bool g3_tensor = false;            // CRT digits on the tensor cores (kernels_g3m.cu)
+  bool g3_tlimbs = false;            // CRT limbs on the tensor cores (kernels_g3l.cu)
   int64_t g3m_x_elems = 0;           // their operand digits
   uint16_t *d_g3m_x = nullptr;
   int64_t *d_g3m_xoff = nullptr;

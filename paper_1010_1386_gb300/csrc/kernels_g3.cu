@@ -24,6 +24,8 @@
 
 namespace {
 
+#include "tcdigits.cuh"  // store_digits8
+
 __device__ __forceinline__ int32_t signed_rep3(uint32_t v, uint32_t p) {
   return v > (p >> 1) ? (int32_t)v - (int32_t)p : (int32_t)v;
 }
@@ -33,188 +35,255 @@ __device__ __forceinline__ uint32_t finish64_3(int64_t s, const ModP &m) {
 }
 
 #define G3T_BK 64  // digits per digit block
-#ifndef RS_G3T_LS16
-#define RS_G3T_LS16 1  // thread groups per 16-coefficient tile (1 or 2)
-#endif
+#define G3T_SB 4   // digits per sub-block
 #define G3T_LC 32  // earlier digits per staged chunk
 
-// Digits by tiles: a block of 256 threads owns JT (32, or 16 when there are
-// few coefficients to spread over the SMs) consecutive coefficients of one
-// pair and produces their digits 64 at a time.  For the digit block
-// [k0, k0 + 64) the contribution of every earlier digit,
+// Digits by tiles: a block owns JT (32, or 16 when there are few coefficients
+// to spread over the SMs) consecutive coefficients of one pair and produces
+// their digits 64 at a time.  For the digit block [k0, k0 + 64) the
+// contribution of every earlier digit,
 //   A[k][j] = sum_{l < k0} W[k][l] v_l(j),
-// is the product of a 64 x k0 slice of W and a k0 x 32 slice of digits:
-// chunks of both are staged in shared memory and each thread accumulates a
-// 4 x JT/16 block lazily in int64 (a fold with its row's 2^32 mod p_k every 7
-// products).  The 64 digits of the block then follow one by one (JT lanes of
-// one warp, lane = coefficient) from the triangle of W inside the block, with the
-// residues, constants and that triangle prefetched into shared memory.
-// The work per coefficient is still K^2 / 2 products, but W and the digits
-// come from shared memory, each value reused 32 and 64 times.
+// is the product of a 64 x k0 slice of W and a k0 x JT slice of digits: chunks
+// of both are staged in shared memory, and each of the 128 threads of a group
+// accumulates 8 rows x JT/16 columns in int64.  |W|, |v| <= (p - 1) / 2, so 8
+// products and a 32-bit rest stay below 2 (p - 1)^2 + 2^32 < 2^63; after every
+// 8 the high words move to sums of their own (adds, while a fold by
+// 2^32 mod p would take the multiply pipe that bounds the loop).  LS groups
+// share the chunks of a block.
+//
+// The digits of the block then follow from the triangle of W inside it, with
+// the constants folded in: S_k = (r_k - A[k]) c_k R, congruent to v_k R,
+// W'[k][l] = -c_k W[k][l] (a table of 64 x 64 blocks, laid out as it is used)
+// and h_k = (p_k - 1) / 2 give
+//   v_k + h_k = REDC(S_k + h_k R + sum_{k0 <= l < k} W'[k][l] v_l)  in [0, p_k),
+// so a digit waits for one REDC and one subtraction (about 45 cycles).  The 16
+// threads that hold rows 4 s .. 4 s + 3 take the four digits of sub-block s in
+// registers, right-looking; after a barrier the threads of later rows add
+// these digits to their own sums (4 products and a fold per sum, independent;
+// W' is loaded before the barrier).  Four digits a step, because the additions
+// to eight rows a thread took longer than eight digits' chain.
+// The block's residues, triangle and constants are copied to shared memory
+// while its chunks are multiplied.
+//
+// What bounds it: this chain with few primes (before, one warp took all 64
+// digits left-looking, 2,000 dependent product steps a block), the products
+// with many.  Measured, before and now: see the choice of the digit kernels in
+// engine.cu.
+__device__ __forceinline__ void copy_async4(void *dst, const void *src) {
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src)
+               : "memory");
+}
+__device__ __forceinline__ void copy_async16(void *dst, const void *src) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src)
+               : "memory");
+}
+
 template <int JT, int LS>
-__global__ void __launch_bounds__(256 * LS, 4 / LS) g3t_kernel(G3Args a) {
+__global__ void __launch_bounds__(128 * LS, 4 / LS) g3t_kernel(G3Args a) {
   constexpr int CJ = JT / 16;  // columns per thread
-  // LS thread groups of 256 share the earlier-digit chunks of a digit block
-  // (group q takes chunks q, q + LS, ...) and their partial sums are added
-  // through shared memory; with few tiles per SM this multiplies the warps
-  // without changing each thread's 4 x CJ register block.
-  // W[k0 + r][l0 + c] at Ws[q][c][r]: rows of 68 words keep each thread's four
-  // consecutive r 16-byte aligned, so they come in one shared load
+  // W[k0 + r][l0 + c] at Ws[.][c][r]: rows of 68 words keep eight consecutive r
+  // 16-byte aligned (two shared loads) and the staging stores free of conflicts
   __shared__ __align__(16) int32_t Ws[LS][G3T_LC][G3T_BK + 4];
-  __shared__ int32_t Vs[LS][G3T_LC][JT];                        // digit l0 + c of coefficient j0 + jj
-  __shared__ int32_t Wt[G3T_BK][G3T_BK + 1];                    // W[k0 + r][k0 + c], c < r
-  __shared__ uint32_t Ds[G3T_BK][JT];                           // r_k(j) - A[k][j] mod p_k
-  __shared__ int32_t Vb[G3T_BK][JT];                            // the block's digits
+  __shared__ int32_t Vs[LS][G3T_LC][JT];                                 // digit l0 + c of coefficient j0 + jj
+  __shared__ __align__(16) int32_t Wt[G3T_BK / G3T_SB][G3T_BK][G3T_SB];  // W'[k0 + r][k0 + 4 s + i], 4 s + i < r
+  __shared__ int32_t Vb[G3T_BK][JT];                                     // the block's residues, then its digits
   __shared__ ModP Ms[G3T_BK];
   __shared__ uint32_t Cs[G3T_BK];
-  static_assert(LS == 1 || (size_t)(LS - 1) * 256 * 4 * CJ * 8 <= sizeof(Ws), "partial sums fit in Ws");
+  constexpr int R = 8 / LS;  // rows per thread in the triangle: 8 rg + R grp + i
+  static_assert(LS <= 2 && (LS == 1 || G3T_BK * JT * 8 <= (int)sizeof(Ws)), "the groups' sums fit in Ws");
   const int2 task = a.tasks[blockIdx.x];
   const PairDesc pd = a.pairs[task.x];
   const int K = pd.K, N = pd.N, S = pd.NI, j0 = task.y, tid = threadIdx.x;
-  const int grp = tid >> 8, ltid = tid & 255;
-  const int rg = ltid >> 4, cg = ltid & 15;  // rows 4 rg .. 4 rg + 3, columns CJ cg .. CJ cg + CJ - 1
+  const int grp = tid >> 7, ltid = tid & 127, warp = ltid >> 5, lane = ltid & 31;
+  const int rg = ltid >> 4, cg = ltid & 15;  // rows 8 rg .. 8 rg + 7, columns CJ cg .. CJ cg + CJ - 1
   uint32_t *col = a.coef + pd.img_off;       // residue, then digit, of (k, j) at col[k S + j]
+  auto group_sync = [&] { asm volatile("bar.sync %0, 128;" ::"r"(grp + 1) : "memory"); };
   for (int k0 = 0; k0 < K; k0 += G3T_BK) {
     const int bk = min(G3T_BK, K - k0);
-    for (int r = tid; r < bk; r += blockDim.x) {
-      Ms[r] = a.mods[k0 + r];
-      Cs[r] = a.crt[k0 + r];
-    }
-    __syncthreads();
-    uint32_t c32[4];
-#pragma unroll
-    for (int i = 0; i < 4; ++i) c32[i] = 4 * rg + i < bk ? Ms[4 * rg + i].r1 : 0u;
-    int64_t acc[4][CJ];
-#pragma unroll
-    for (int i = 0; i < 4; ++i)
-#pragma unroll
-      for (int c = 0; c < CJ; ++c) acc[i][c] = 0;
-    // Chunks of W (8 values per thread) and digits are loaded into registers
-    // one chunk ahead, so their latency overlaps the products.
-    constexpr int NW = G3T_LC * G3T_BK / 256, NV = G3T_LC * JT / 256;
+    // Chunks of W (16 rows of one column per thread) and digits are loaded into
+    // registers one chunk ahead, so their latency overlaps the products.
+    constexpr int NW = 16, NV = G3T_LC * JT / 128;
     int32_t wreg[NW], vreg[NV];
+    const int wk = k0 + 16 * warp;  // the triangle of W has fewer than 2^27 entries (K <= 16384)
+    const int32_t *wrow = a.wtab + wk * (wk - 1) / 2 + lane;
+    const uint32_t *vcol = col + (size_t)(ltid / JT) * S + j0 + ltid % JT;
+    const bool vlive = j0 + ltid % JT < N;
     auto fetch = [&](int l0) {
 #pragma unroll
-      for (int q = 0; q < NW; ++q) {
-        const int e = ltid + 256 * q, r = e >> 5, c = e & 31, k = k0 + r;
-        wreg[q] = r < bk ? __ldg(a.wtab + (size_t)k * (k - 1) / 2 + l0 + c) : 0;
-      }
+      for (int q = 0; q < NW; ++q)  // row wk + q starts q wk + q (q - 1) / 2 after row wk
+        wreg[q] = wk + q < K ? __ldg(wrow + (l0 + q * wk + q * (q - 1) / 2)) : 0;
 #pragma unroll
-      for (int q = 0; q < NV; ++q) {
-        const int e = ltid + 256 * q, c = e / JT, jj = e % JT, j = j0 + jj;
-        vreg[q] = j < N ? (int32_t)col[(size_t)(l0 + c) * S + j] : 0;
-      }
+      for (int q = 0; q < NV; ++q) vreg[q] = vlive ? (int32_t)vcol[(size_t)(l0 + q * (128 / JT)) * S] : 0;
     };
     const int nch = k0 / G3T_LC;  // k0 is a multiple of G3T_LC: full chunks
     if (grp < nch) fetch(grp * G3T_LC);
-    for (int it = 0; it * LS < nch; ++it) {
-      const int ch = it * LS + grp, l0 = ch * G3T_LC;
-      const bool act = ch < nch;
-      if (act) {
+    const int32_t *tri = a.wtri + (size_t)(k0 / G3T_BK) * (G3T_BK * G3T_BK);
 #pragma unroll
-        for (int q = 0; q < NW; ++q) {
-          const int e = ltid + 256 * q;
-          Ws[grp][e & 31][e >> 5] = wreg[q];
-        }
+    for (int e = tid; e < G3T_BK * G3T_BK / 4; e += 128 * LS) {  // piece (s, r): not all zero, and used
+      const int r = e & 63;
+      if (r < bk && r > 4 * (e >> 6)) copy_async16(&Wt[e >> 6][r][0], tri + 4 * e);
+    }
 #pragma unroll
-        for (int q = 0; q < NV; ++q) {
-          const int e = ltid + 256 * q;
-          Vs[grp][e / JT][e % JT] = vreg[q];
-        }
-      }
-      __syncthreads();
-      if (ch + LS < nch) fetch(l0 + LS * G3T_LC);
-      if (act) {
-        // |acc| < 2^53 after a fold and each product is below 2^60 in size, so
-        // 7 products may follow a fold: four groups of 7 steps and one of 4.
-        auto steps = [&](int c0, int n) {
+    for (int e = tid; e < G3T_BK * JT; e += 128 * LS)
+      if (e / JT < bk && j0 + e % JT < N) copy_async4(&Vb[e / JT][e % JT], col + (size_t)(k0 + e / JT) * S + j0 + e % JT);
+    if (tid < G3T_BK) {  // rows past the last prime repeat it; their sums are never used
+      copy_async16(&Ms[tid], a.mods + (k0 + min(tid, bk - 1)));
+      copy_async4(&Cs[tid], a.crt + (k0 + min(tid, bk - 1)));
+    }
+    int64_t acc[8][CJ], high[8][CJ];
 #pragma unroll
-          for (int c = c0; c < c0 + 7; ++c) {
-            if (c - c0 >= n) break;
-            const int4 w4 = *reinterpret_cast<const int4 *>(&Ws[grp][c][4 * rg]);
-            const int32_t w[4] = {w4.x, w4.y, w4.z, w4.w};
-            int32_t v[CJ];
+    for (int i = 0; i < 8; ++i)
 #pragma unroll
-            for (int cc = 0; cc < CJ; ++cc) v[cc] = Vs[grp][c][CJ * cg + cc];
+      for (int c = 0; c < CJ; ++c) acc[i][c] = high[i][c] = 0;
+    for (int ch = grp; ch < nch; ch += LS) {
 #pragma unroll
-            for (int i = 0; i < 4; ++i)
+      for (int q = 0; q < NW; q += 4)
+        *reinterpret_cast<int4 *>(&Ws[grp][lane][16 * warp + q]) =
+            make_int4(wreg[q], wreg[q + 1], wreg[q + 2], wreg[q + 3]);
 #pragma unroll
-              for (int cc = 0; cc < CJ; ++cc) acc[i][cc] = rs_mac_s32(acc[i][cc], w[i], v[cc]);
-          }
-#pragma unroll
-          for (int i = 0; i < 4; ++i)
-#pragma unroll
-            for (int cc = 0; cc < CJ; ++cc) acc[i][cc] = rs_fold64(acc[i][cc], c32[i]);
-        };
+      for (int q = 0; q < NV; ++q) Vs[grp][(ltid + 128 * q) / JT][ltid % JT] = vreg[q];
+      group_sync();
+      if (ch + LS < nch) fetch((ch + LS) * G3T_LC);
+      if (16 * warp < bk) {
 #pragma unroll 1
-        for (int c0 = 0; c0 < 28; c0 += 7) steps(c0, 7);
-        steps(28, G3T_LC - 28);
-      }
-      __syncthreads();
-    }
-    if constexpr (LS > 1) {  // the other groups' partial sums, through the (now unused) staging buffer
-      int64_t *part = reinterpret_cast<int64_t *>(&Ws[0][0][0]);
-      if (grp > 0) {
+        for (int c0 = 0; c0 < G3T_LC; c0 += 8) {
 #pragma unroll
-        for (int i = 0; i < 4; ++i)
+          for (int c = 0; c < 8; ++c) {
+            const int4 lo = *reinterpret_cast<const int4 *>(&Ws[grp][c0 + c][8 * rg]);
+            const int4 hi = *reinterpret_cast<const int4 *>(&Ws[grp][c0 + c][8 * rg + 4]);
+            const int32_t w[8] = {lo.x, lo.y, lo.z, lo.w, hi.x, hi.y, hi.z, hi.w};
 #pragma unroll
-          for (int c = 0; c < CJ; ++c)
-            part[(((size_t)(grp - 1) * 256 + ltid) * 4 + i) * CJ + c] = rs_fold64(acc[i][c], c32[i]);
-      }
-      __syncthreads();
-      if (grp == 0) {
+            for (int cc = 0; cc < CJ; ++cc) {
+              const int64_t v = Vs[grp][c0 + c][CJ * cg + cc];
 #pragma unroll
-        for (int i = 0; i < 4; ++i)
-#pragma unroll
-          for (int c = 0; c < CJ; ++c) {
-            int64_t sum = rs_fold64(acc[i][c], c32[i]);  // |.| < 2^53 each: LS of them stay below 2^63
-            for (int q = 1; q < LS; ++q) sum += part[(((size_t)(q - 1) * 256 + ltid) * 4 + i) * CJ + c];
-            acc[i][c] = sum;
+              for (int i = 0; i < 8; ++i) acc[i][cc] += w[i] * v;
+            }
           }
-      }
-    }
-    // D = r - A mod p_k (plain: W is in Montgomery form, the finish removes R)
-    if (grp == 0) {
 #pragma unroll
-      for (int i = 0; i < 4; ++i) {
-        const int r = 4 * rg + i;
-        if (r >= bk) continue;
-        const ModP m = Ms[r];
+          for (int i = 0; i < 8; ++i)
 #pragma unroll
-        for (int c = 0; c < CJ; ++c) {
-          const int jj = CJ * cg + c, j = j0 + jj;
-          const uint32_t tA = finish64_3(rs_fold64(acc[i][c], m.r1), m);
-          const uint32_t res = j < N ? col[(size_t)(k0 + r) * S + j] : 0u;
-          Ds[r][jj] = msub(res, tA, m.p);
+            for (int cc = 0; cc < CJ; ++cc) {
+              high[i][cc] += (int32_t)(acc[i][cc] >> 32);
+              acc[i][cc] = (uint32_t)acc[i][cc];
+            }
         }
       }
+      group_sync();
     }
-    for (int e = tid; e < G3T_BK * G3T_BK; e += blockDim.x) {
-      const int r = e >> 6, c = e & 63, k = k0 + r;
-      Wt[r][c] = (c < r && r < bk) ? __ldg(a.wtab + (size_t)k * (k - 1) / 2 + k0 + c) : 0;
-    }
+    asm volatile("cp.async.wait_all;" ::: "memory");
     __syncthreads();
-    if (tid < JT) {  // the block's digits in order, lane = coefficient
-      const int jj = tid, j = j0 + jj;
-      for (int r = 0; r < bk; ++r) {
-        const ModP m = Ms[r];
-        int64_t s0 = 0, s1 = 0;
-        int n = 0;
-        for (int c = 0; c + 1 < r; c += 2) {
-          s0 = rs_mac_s32(s0, Wt[r][c], Vb[c][jj]);
-          s1 = rs_mac_s32(s1, Wt[r][c + 1], Vb[c + 1][jj]);
-          if (++n == 7) {
-            s0 = rs_fold64(s0, m.r1);
-            s1 = rs_fold64(s1, m.r1);
-            n = 0;
+    // acc + 2^32 high, |high| < 2^42, congruent to a word below 2^56
+#pragma unroll
+    for (int i = 0; i < 8; ++i) {
+      const uint32_t c32 = Ms[8 * rg + i].r1;
+#pragma unroll
+      for (int cc = 0; cc < CJ; ++cc) acc[i][cc] += rs_fold64(high[i][cc], c32) * (int64_t)c32;
+    }
+    int64_t sum[R][CJ];
+    if constexpr (LS > 1) {  // each group keeps R of a thread's rows; the others' sums go through the staging buffer
+      int64_t *part = reinterpret_cast<int64_t *>(&Ws[0][0][0]);
+#pragma unroll
+      for (int i = 0; i < R; ++i)
+#pragma unroll
+        for (int cc = 0; cc < CJ; ++cc) {
+          part[((grp * R + i) * CJ + cc) * 128 + ltid] = grp ? acc[i][cc] : acc[R + i][cc];
+          sum[i][cc] = grp ? acc[R + i][cc] : acc[i][cc];
+        }
+      __syncthreads();
+#pragma unroll
+      for (int i = 0; i < R; ++i)
+#pragma unroll
+        for (int cc = 0; cc < CJ; ++cc) sum[i][cc] += part[(((1 - grp) * R + i) * CJ + cc) * 128 + ltid];
+    } else {
+#pragma unroll
+      for (int i = 0; i < R; ++i)
+#pragma unroll
+        for (int cc = 0; cc < CJ; ++cc) sum[i][cc] = acc[i][cc];
+    }
+    // S + h R: (r - A) c R (plain r: W is in Montgomery form, its REDC removes R;
+    // c in Montgomery form brings R back) as a folded word, plus h R mod p
+    const int row0 = 8 * rg + R * grp;
+    uint32_t rp[R], rpi[R], rc[R];
+#pragma unroll
+    for (int i = 0; i < R; ++i) {
+      const int r = row0 + i;
+      const ModP m = Ms[r];
+      const uint32_t c = Cs[r], hR = to_mont(m.p >> 1, m);
+      rp[i] = m.p;
+      rpi[i] = m.pinv;
+      rc[i] = m.r1;
+#pragma unroll
+      for (int cc = 0; cc < CJ; ++cc) {
+        const uint32_t res = r < bk && j0 + CJ * cg + cc < N ? (uint32_t)Vb[r][CJ * cg + cc] : 0u;
+        const uint32_t A = redc((uint64_t)(sum[i][cc] + ((int64_t)m.p << 27)), m.p, m.pinv);  // |sum| < 2^57
+        sum[i][cc] = rs_fold64((int64_t)((uint64_t)msub(res, A, m.p) * c), m.r1) + hR;
+      }
+    }
+    __syncthreads();  // the residues in Vb are read: the digits take their place
+    const int nsb = (bk + 3) / 4;
+    for (int s = 0; s < nsb; ++s) {
+#pragma unroll
+      for (int q = 0; q < R; q += 4) {
+        if (row0 + q != 4 * s) continue;
+        int32_t w[4][4];  // w[r][i], i < r: W' of the sub-block's triangle
+#pragma unroll
+        for (int r = 1; r < 4; ++r) {
+          const int4 x = *reinterpret_cast<const int4 *>(&Wt[s][4 * s + r][0]);
+          w[r][0] = x.x, w[r][1] = x.y, w[r][2] = x.z;
+        }
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+#pragma unroll
+          for (int cc = 0; cc < CJ; ++cc) {
+            // |sum| < 2^57 + 3 (p/2)^2: p 2^32 more if negative leaves [0, p 2^32)
+            const uint32_t p = rp[q + i], h = (uint32_t)((uint64_t)sum[q + i][cc] >> 32);
+            const uint32_t z = redc(((uint64_t)rs_umin(h, h + p) << 32) | (uint32_t)sum[q + i][cc], p, rpi[q + i]);
+            const int32_t vs = (int32_t)z - (int32_t)(p >> 1);
+#pragma unroll
+            for (int r = i + 1; r < 4; ++r) sum[q + r][cc] += (int64_t)w[r][i] * vs;
+            Vb[4 * s + i][CJ * cg + cc] = vs;
           }
         }
-        if (r & 1) s0 = rs_mac_s32(s0, Wt[r][r - 1], Vb[r - 1][jj]);
-        const int64_t s = rs_fold64(rs_fold64(s0, m.r1) + rs_fold64(s1, m.r1), m.r1);
-        const uint32_t v = mmul(msub(Ds[r][jj], finish64_3(s, m), m.p), Cs[r], m);
-        const int32_t vs = signed_rep3(v, m.p);
-        Vb[r][jj] = vs;
-        if (j < N) col[(size_t)(k0 + r) * S + j] = (uint32_t)vs;
+      }
+      int4 w4[R];
+#pragma unroll
+      for (int i = 0; i < R; ++i) w4[i] = *reinterpret_cast<const int4 *>(&Wt[s][row0 + i][0]);
+      __syncthreads();
+      if (row0 + R > 4 * s + 4) {  // the later rows' sums, 4 products below (p/2)^2 each, folded
+        int32_t v[4][CJ];
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+#pragma unroll
+          for (int cc = 0; cc < CJ; ++cc) v[i][cc] = Vb[4 * s + i][CJ * cg + cc];
+#pragma unroll
+        for (int i = 0; i < R; ++i) {
+          if (R > 4 && row0 + i < 4 * s + 4) continue;
+#pragma unroll
+          for (int cc = 0; cc < CJ; ++cc) {
+            int64_t t = (int64_t)w4[i].x * v[0][cc];
+            t += (int64_t)w4[i].y * v[1][cc];
+            t += (int64_t)w4[i].z * v[2][cc];
+            t += (int64_t)w4[i].w * v[3][cc];
+            sum[i][cc] += rs_fold64(t, rc[i]);
+          }
+        }
+      }
+    }
+    // the digits over the residues (the last sub-block's barrier is behind)
+#pragma unroll
+    for (int e = tid; e < G3T_BK * JT; e += 128 * LS) {
+      const int r = e / JT, j = j0 + e % JT;
+      if (r < bk && j < N) col[(size_t)(k0 + r) * S + j] = (uint32_t)Vb[r][e % JT];
+    }
+    if (a.xdig) {  // and as operand digits of the tensor-core limb kernel
+      uint16_t *x = a.xdig + pd.xd_off + (int64_t)(j0 >> 7) * ((K + 63) / 64) * 32768;
+      for (int e = tid; e < G3T_BK / 8 * JT; e += 128 * LS) {
+        const int r = 8 * (e / JT), jj = e % JT;
+        if (r >= bk || j0 + jj >= N) continue;
+        int32_t v[8];
+#pragma unroll
+        for (int i = 0; i < 8; ++i) v[i] = r + i < bk ? Vb[r + i][jj] : 0;
+        store_digits8(x, (j0 & 127) + jj, k0 + r, v);
       }
     }
     __syncthreads();  // this block's digits are read by the next digit blocks
@@ -482,6 +551,23 @@ __global__ void crt_w_kernel(const ModP *mods, int K, int32_t *wtab) {
   }
 }
 
+// The triangle of W inside each 64-prime block with -c_k folded in, as the
+// tiled digit kernel copies it: -c_k W[k][l] (Montgomery form, signed) for
+// k = 64 b + r, l = 64 b + 4 s + i < k at [b][s][r][i], zero elsewhere.
+__global__ void crt_tri_kernel(const ModP *mods, const uint32_t *crt, const int32_t *wtab, int K, int32_t *wtri) {
+  const int b = blockIdx.x;
+  for (int e = threadIdx.x; e < G3T_BK * G3T_BK; e += blockDim.x) {
+    const int s = e >> 8, r = (e >> 2) & 63, c = 4 * s + (e & 3), k = G3T_BK * b + r;
+    int32_t w = 0;
+    if (c < r && k < K) {
+      const ModP m = mods[k];
+      const int32_t x = wtab[(size_t)k * (k - 1) / 2 + G3T_BK * b + c];
+      w = signed_rep3(mmul(x < 0 ? (uint32_t)(-x) : m.p - (uint32_t)x, crt[k], m), m.p);
+    }
+    wtri[(size_t)b * (G3T_BK * G3T_BK) + e] = w;
+  }
+}
+
 // One warp per (factor, prime): g mod p by Horner over g's limbs
 // (r <- r 2^32 + limb, with 2^32 = R mod p taken as mmul by R^2 mod p), its
 // inverse by Fermat, then the factor's residues times that inverse (plain
@@ -521,9 +607,9 @@ cudaError_t launch_g3t(int nt, const G3Args &a, const int2 *ttasks, cudaStream_t
   at.tasks = ttasks;
   if (nt) {
     if (jt == 16)
-      g3t_kernel<16, RS_G3T_LS16><<<nt, 256 * RS_G3T_LS16, 0, s>>>(at);
+      g3t_kernel<16, 2><<<nt, 256, 0, s>>>(at);
     else
-      g3t_kernel<32, 1><<<nt, 256, 0, s>>>(at);
+      g3t_kernel<32, 1><<<nt, 128, 0, s>>>(at);
   }
   return cudaGetLastError();
 }
@@ -545,7 +631,13 @@ cudaError_t launch_g3bc(int nb, int nc, const G3Args &a, const int2 *otasks, cud
   return cudaGetLastError();
 }
 
-cudaError_t launch_crt_tables(const ModP *mods, int K, int32_t *wtab, cudaStream_t s) {
+int64_t crt_tri_words(int K) { return (int64_t)((K + G3T_BK - 1) / G3T_BK) * (G3T_BK * G3T_BK); }
+
+cudaError_t launch_crt_tables(const ModP *mods, const uint32_t *crt, int K, int32_t *wtab, int32_t *wtri,
+                              cudaStream_t s) {
   crt_w_kernel<<<(K + 63) / 64, 64, 0, s>>>(mods, K, wtab);
+  cudaError_t e = cudaGetLastError();
+  if (e != cudaSuccess) return e;
+  crt_tri_kernel<<<(K + G3T_BK - 1) / G3T_BK, 256, 0, s>>>(mods, crt, wtab, K, wtri);
   return cudaGetLastError();
 }

@@ -38,6 +38,7 @@ struct PairDesc {
   int64_t out_off;       // offset of the N*Lout output block (coefficient-major)
   int64_t xl_off;        // offset of the CRT digit scratch: N * 16 * ceil(Lout/16) words
   int64_t cy_off;        // offset of the CRT chunk carries: N * ceil(Lout/16) int64
+  int64_t xd_off;        // element offset of the operand digits of its first 128 coefficients
 };
 
 // G1 work item: point pairs [x0, x0 + n) of one (pair, prime), two threads
@@ -155,12 +156,8 @@ struct G2tArgs {
 
 #define RS_G2T_MAX_M 4096  // point pairs per (pair, prime) the tensor-core form takes
 
-#ifndef RS_G3M_MIN_K
-#define RS_G3M_MIN_K 128  // largest prime count from which a batch's digits take the tensor cores
-#endif
-#ifndef RS_G3M_WIDE_K
-#define RS_G3M_WIDE_K 1024  // ... and from which they do so even with few coefficient tiles
-#endif
+#define RS_G3M_MIN_K 128  // largest prime count from which a batch's digits may take the tensor cores
+#define RS_G3L_MIN_K 24   // ... and from which its limbs do
 
 // Tensor-core CRT digits (kernels_g3m.cu): one block per 128 coefficients of
 // one pair (the output kernel's tasks), over 64-prime digit blocks.
@@ -246,10 +243,12 @@ struct G3Args {
   const ModP *mods;
   const uint32_t *crt;     // (p_0 ... p_{k-1})^{-1} mod p_k, Montgomery form
   const int32_t *wtab;     // triangular: W[k][l] = p_0 ... p_{l-1} mod p_k (Montgomery, signed)
+  const int32_t *wtri;     // its 64 x 64 diagonal blocks times -c_k (the tiled digit kernel)
   const uint16_t *p16;     // prefix products p_0 ... p_{k-1} in 16-bit digits
   const int32_t *poff;     // row offsets into p16 (u16 units, multiples of 32)
   const int32_t *nh;       // digits of each prefix product
   uint32_t *coef;          // in: R mod p_k (plain); overwritten by mixed-radix digits
+  uint16_t *xdig = nullptr;  // the tiled digit kernel writes the digits here too, as operand digits (NULL: not)
   uint32_t *xl;            // 16-bit digit pairs of R_j, [16 chunk + w][N] per pair
   int64_t *carry;          // chunk carries [chunk][N] per pair
   uint32_t *out;           // out: [coefficient][limb]
@@ -296,11 +295,9 @@ cudaError_t launch_g3t(int nt, const G3Args &a, const int2 *ttasks, cudaStream_t
 // CRT digits with one thread per coefficient (tasks: (pair, first
 // coefficient) per block of 128 coefficients, the output kernel's tasks).
 cudaError_t launch_g3p(int nt, const G3Args &a, const int2 *tasks, cudaStream_t s);
-// Coefficients per SM from which a batch takes the one-thread-per-coefficient
-// digit kernel.
-#ifndef RS_G3P_MIN_COEF_PER_SM
+// Coefficients per SM from which a batch of any prime count takes the
+// one-thread-per-coefficient digit kernel.
 #define RS_G3P_MIN_COEF_PER_SM 1024
-#endif
 cudaError_t launch_yun(int ntasks, const YunArgs &a, cudaStream_t s);
 // Schur variant of G1: one block per tile, `slots` = ceil((m_y + n_y) / 32)
 // over the batch, smem = staged residues of the largest pair; then the
@@ -319,7 +316,9 @@ struct ScaleDesc {
 };
 cudaError_t launch_scale(const ScaleDesc *sd, int nf, int kmax, const ModP *mods, const uint32_t *gw,
                          const uint32_t *in, uint32_t *out, cudaStream_t s);
-cudaError_t launch_crt_tables(const ModP *mods, int K, int32_t *wtab, cudaStream_t s);
+int64_t crt_tri_words(int K);  // words of the block triangles for K primes
+cudaError_t launch_crt_tables(const ModP *mods, const uint32_t *crt, int K, int32_t *wtab, int32_t *wtri,
+                              cudaStream_t s);
 cudaError_t launch_init_primes(const uint32_t *primes, int n, ModP *mods, uint32_t *vtab,
                                uint32_t *crt, uint32_t *qbase, cudaStream_t s);
 cudaError_t launch_tables(const ModP *mods, const uint32_t *qbase, int K, int N, int stride,

@@ -770,6 +770,7 @@ extern "C" int rs_squarefree_batch(rs_ctx *ctx, int32_t n, const rs_bipoly *f, c
         a3.mods = ctx->d_mods;
         a3.crt = ctx->d_crt;
         a3.wtab = tab.wtab;
+        a3.wtri = tab.wtri;
         a3.p16 = tab.p16;
         a3.poff = tab.poff;
         a3.nh = tab.nh;
@@ -942,6 +943,7 @@ extern "C" int rs_squarefree_batch(rs_ctx *ctx, int32_t n, const rs_bipoly *f, c
         a3.mods = ctx->d_mods;
         a3.crt = ctx->d_crt;
         a3.wtab = tab.wtab;
+        a3.wtri = tab.wtri;
         a3.p16 = tab.p16;
         a3.poff = tab.poff;
         a3.nh = tab.nh;
