@@ -24,6 +24,12 @@ __device__ __forceinline__ void block_scan_mul(uint32_t v, uint32_t &pre, uint32
   uint32_t es = __shfl_down_sync(0xffffffffu, is, 1);
   if (lane == 0) ep = m.r1;
   if (lane == 31) es = m.r1;
+  if (nw == 1) {
+    pre = ep;
+    suf = es;
+    total = __shfl_sync(0xffffffffu, ip, 31);
+    return;
+  }
   if (lane == 31) scratch[warp] = ip;
   __syncthreads();
   if (warp == 0) {
@@ -53,8 +59,9 @@ __device__ __forceinline__ void block_scan_mul(uint32_t v, uint32_t &pre, uint32
 
 // out[i] = d[i]^{-1} for i < n (Montgomery's simultaneous inversion: one
 // Fermat inverse of the product, prefix and suffix products for the rest).
+// d in Montgomery form; out too, or plain.
 __device__ void batch_invert(const uint32_t *d, uint32_t *out, int n, const ModP &m,
-                             uint32_t *scratch) {
+                             uint32_t *scratch, bool plain = false) {
   const int T = blockDim.x;
   const int E = (n + T - 1) / T;
   const int beg = min((int)threadIdx.x * E, n), end = min(beg + E, n);
@@ -62,7 +69,8 @@ __device__ void batch_invert(const uint32_t *d, uint32_t *out, int n, const ModP
   for (int i = beg; i < end; ++i) v = mmul(v, d[i], m);
   uint32_t pre, suf, total;
   block_scan_mul(v, pre, suf, total, m, scratch);
-  const uint32_t itot = minv(total, m);
+  uint32_t itot = minv(total, m);
+  if (plain) itot = from_mont(itot, m);
   uint32_t r = pre;
   for (int i = beg; i < end; ++i) {
     out[i] = r;

@@ -201,15 +201,58 @@ int rs_g2_len(int N) {
   return lg <= RS_NTT_LGMAX ? lg : 0;
 }
 
-// Cost per (pair, prime) in direct multiply-accumulate-equivalents of issue
-// time: a direct multiply-accumulate issues about 3.8 instructions (two
-// convolutions of N^2 / 2 each); the transform form takes 12 transforms of
-// (L/2) lg radix-4 butterflies, which timed at about 6.5 such units each on
-// GB300 (lengths 2^9 and 2^10 ran 1.08x and 1.44x faster than direct).
+// Cost per (pair, prime) of interpolating N point pairs, in units of 0.37 ps of
+// the whole GPU.  Direct: one unit per N^2 (two multiply-accumulates) and 170
+// per point for the rest of the kernel (12 ns at N = 113, 1.56 us at 2,049).
+// Transforms: 12 of (L/2) lg radix-4 butterflies, 6.5 units each (1.60 us at
+// N = 2,049, L = 2^13).
 double rs_g2_cost(int N, int form) {
   const int lg = rs_g2_len(N);
-  if (form == 0 || lg == 0) return 3.8 * (double)N * N;
+  if (form == 0 || lg == 0) return (double)N * N + 170.0 * N;
   return 12.0 * 6.5 * (double)(1 << (lg - 1)) * lg + 60.0 * N;
+}
+
+// Launch shape of the direct form for M point pairs: the threads of a block,
+// the segments of a block pair's walk, the halves (E, O) at once, and whether
+// E and O get a block each (a cluster of two); see g2_kernel.  The least of an
+// estimate in cycles of the busiest SM, fitted to sweeps over 32 to 512
+// threads: a warp's step (one chunk, 56 wide products) takes 277 cycles of its
+// scheduler, or 622 from start to end alone; the rest of a block 1,900 per warp
+// and 550 per warp, half and round over the points, and 5,000 from start to
+// end.  Measured (us, G2 stage): 40,000 tasks of M = 113: 427 with 32 threads
+// (2 rounds, 3 segments), 474, 597, 986 and 1,599 with 64, 128, 256 and 512;
+// 546 of 2,049: 1,140, 1,027, 984 and 853 with 64, 128, 256 and 512; 69 of 451:
+// 20.2 with 384 threads in clusters, 24.2 with the best single blocks.
+RsG2Shape rs_g2_shape(int M, int64_t tasks, int sms, const RsG2Shape *like) {
+  static const int kT[8] = {32, 64, 96, 128, 192, 256, 384, 512};
+  const int nblk = (M + RS_CONV_R - 1) / RS_CONV_R, npair = (nblk + 1) / 2, W = M + 2 * RS_G2_PAD;
+  RsG2Shape best{256, 1, 1, 0, (size_t)(3 * W + M) * 4};
+  double tbest = 1e300;
+  for (int split = 0; split < 2; ++split) {
+    if (like && split != like->split) continue;
+    const int nh = split ? 1 : 2;
+    const int64_t n = ((tasks << split) + sms - 1) / sms;  // blocks of the busiest SM
+    if (split && n > 4 && !like) continue;
+    for (int T : kT) {
+      if (like && T != like->threads) continue;
+      for (int rounds = 1; rounds <= 2; ++rounds) {
+        const int S = std::max(1, std::min(std::min(nblk + 1, 16), rounds * T / (nh * npair)));
+        const size_t smem = (size_t)((nh + 1) * W + S * nh * M) * 4;
+        if (smem > (size_t)RS_G2_MAX_SMEM_BYTES) continue;
+        const int len = (nblk + S) / S, units = nh * npair * S, iters = (M + T - 1) / T;
+        const int64_t res = std::max<int64_t>(1, std::min<int64_t>(std::min(32, 1024 / T), (226 * 1024) / (smem + 1536)));
+        const double rest = 550.0 * nh * iters;
+        const double busy = n * 0.25 * (2.0 * len * ((units + 31) / 32) * 277.0 + T / 32 * (1900.0 + rest));
+        const double path = ((n + res - 1) / res) * (2.0 * len * ((units + T - 1) / T) * 622.0 + 5000.0 + rest);
+        const double t = busy * busy + 4.0 * path * path;
+        if (t < tbest) {
+          tbest = t;
+          best = RsG2Shape{T, S, nh, split, smem};
+        }
+      }
+    }
+  }
+  return best;
 }
 
 int rs_ensure_bhat(rs_ctx *ctx, int lg, int K) {
@@ -805,24 +848,46 @@ int rs_build_batch(rs_ctx *ctx, int n, const rs_bipoly *f, const rs_bipoly *g,
     b->g2cls.push_back(gc);
   }
   const int nlg = (int)b->g2cls.size();
-  for (int c = 0; c < 8 && !g2tri; ++c) {
-    RsG2Class gc;
-    gc.threads = 32 * (c + 1);
-    gc.off = (int64_t)g2.size();
-    int cmaxN = 0;
-    for (int i : byN) {
-      const PairPlan &p = b->plans[i];
-      if (g2lg[i] || g2t_lg[i]) continue;
-      const int npair = (((p.N + 1) / 2 + RS_CONV_R - 1) / RS_CONV_R + 1) / 2;  // output-block pairs
-      const int rounds = (npair + 255) / 256;
-      const int warps = (npair + 32 * rounds - 1) / (32 * rounds);
-      if (warps - 1 != c) continue;
-      cmaxN = std::max(cmaxN, (p.N + 1) / 2);
-      for (int k = 0; k < p.K; ++k) g2.push_back(make_int2(b->dev_index[i], k));
+  if (!g2tri && !images_only) {
+    double direct = 0.0;  // the direct form's whole work: a shape is chosen as for that work in tasks of its size
+    for (int i : byN)
+      if (!g2lg[i] && !g2t_lg[i]) direct += b->plans[i].K * rs_g2_cost((b->plans[i].N + 1) / 2, 0);
+    for (size_t u = 0; u < byN.size();) {
+      // One launch per octave of point-pair counts, shaped for its largest;
+      // octaves of one shape together.  (A shape for every count of an uneven
+      // batch of 17 pairs gave 16 launches and 0.36 ms; by octaves 0.27.)
+      if (g2lg[byN[u]] || g2t_lg[byN[u]]) {
+        ++u;
+        continue;
+      }
+      const int top = (b->plans[byN[u]].N + 1) / 2;
+      const RsG2Shape sh = rs_g2_shape(top, (int64_t)(direct / rs_g2_cost(top, 0) + 0.5), ctx->sms, nullptr);
+      const RsG2Class *last = (int)b->g2cls.size() > nlg ? &b->g2cls.back() : nullptr;
+      if (!last || last->threads != sh.threads || last->halves != sh.halves || last->split != sh.split) {
+        RsG2Class nc;
+        nc.off = (int64_t)g2.size();
+        nc.threads = sh.threads;
+        nc.halves = sh.halves;
+        nc.split = sh.split;
+        b->g2cls.push_back(nc);
+      }
+      RsG2Class &gc = b->g2cls.back();
+      RsG2Shape cur = sh;
+      int curM = top;
+      for (; u < byN.size(); ++u) {
+        const PairPlan &p = b->plans[byN[u]];
+        if (g2lg[byN[u]] || g2t_lg[byN[u]]) continue;
+        const int M = (p.N + 1) / 2;
+        if (2 * M <= top) break;
+        if (M != curM) cur = rs_g2_shape(M, (int64_t)(direct / rs_g2_cost(M, 0) + 0.5), ctx->sms, &sh);
+        if (cur.halves != sh.halves) break;
+        curM = M;
+        gc.smem = std::max(gc.smem, cur.smem);
+        b->descs[b->dev_index[byN[u]]].g2_seg = cur.seg;
+        for (int k = 0; k < p.K; ++k) g2.push_back(make_int2(b->dev_index[byN[u]], k));
+      }
+      gc.count = (int)((int64_t)g2.size() - gc.off);
     }
-    gc.count = (int)((int64_t)g2.size() - gc.off);
-    gc.smem = (size_t)4 * (cmaxN + 2 * RS_G2_PAD) * 4;
-    if (gc.count > 0 && !images_only) b->g2cls.insert(b->g2cls.begin() + nlg, gc);  // largest point counts first
   }
   // CRT digits in tiles of 32 coefficients; limbs in blocks of 128
   // coefficients by chunks of 16 output limbs.
@@ -919,7 +984,6 @@ int rs_build_batch(rs_ctx *ctx, int n, const rs_bipoly *f, const rs_bipoly *g,
   b->ng3d = images_only ? 0 : (int)g3d.size();
   b->ng3b = images_only ? 0 : (int)g3b.size();
   b->kmax = maxK;
-  b->g2smem = (size_t)4 * (maxM + 2 * RS_G2_PAD) * 4;
   b->info.input_bytes = b->in_words * 4;
   b->info.output_bytes = b->out_words * 4;
   b->info.kernel_launches = (b->schur ? 2 : (int64_t)b->classes.size()) + (int64_t)b->g2cls.size() + (b->ng3d > 0) +
@@ -1107,7 +1171,7 @@ int rs_build_batch(rs_ctx *ctx, int n, const rs_bipoly *f, const rs_bipoly *g,
       ctx->g2t_ready = e2 == cudaSuccess;
     }
     if (rc == RS_OK && !b->g2cls.empty() && !ctx->g2_ready) {
-      cudaError_t e2 = g2_prepare(b->g2smem);
+      cudaError_t e2 = g2_prepare();
       if (e2 != cudaSuccess) rc = rs_fail(ctx, RS_ERR_CUDA, std::string("G2 set-up: ") + cudaGetErrorString(e2));
       ctx->g2_ready = e2 == cudaSuccess;
     }
@@ -1359,6 +1423,8 @@ static int enqueue(rs_batch *b, bool capturing) {
     a2.gtab = tab.gtab;
     a2.btab = tab.btab;
     a2.tab_stride = tab.N;
+    a2.halves = gc.halves;
+    a2.split = gc.split;
     const int j = (int)b->classes.size() + gi;
     cudaError_t fe = cudaSuccess;
     cudaStream_t si = branch_begin(b, 1, gi, s, &fe);

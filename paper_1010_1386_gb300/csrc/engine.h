@@ -125,6 +125,7 @@ struct RsG2Class {
   int64_t t_task_off = 0, t_item_off = 0;  // first task / work item of the class in the batch lists
   int t_ntask = 0, t_nitem = 0, t_maxM = 0;
   int threads = 256;
+  int halves = 1, split = 0;  // direct form: E and O at once / in a block each
   int64_t off = 0;  // first task of the class in the G2 task list
   int count = 0;
   size_t smem = 0;
@@ -167,7 +168,7 @@ struct rs_batch {
   int64_t in_words = 0, img_words = 0, out_words = 0;
   int64_t shape_off = 0;  // word offset of the per-pair result shapes in the output buffer
   int64_t status_off = 0; // word offset of the device status word (0 = every bounded wait completed)
-  int ng2 = 0, ng3 = 0, g2_threads = 256;
+  int ng2 = 0, ng3 = 0;
   int ng3d = 0, ng3b = 0, kmax = 0;  // CRT digit tiles, limb chunks, largest K
   int g3_jt = 32;                    // coefficients per CRT digit tile (32 or 16)
   bool g3_perthread = false;         // CRT digits with one thread per coefficient
@@ -191,7 +192,6 @@ struct rs_batch {
   uint32_t *d_g2t_y = nullptr;
   int64_t g2t_x_elems = 0;
   int64_t *d_cy = nullptr;
-  size_t g2smem = 0;
   void *arena = nullptr;  // one device allocation carved into the buffers below
   uint32_t *d_in = nullptr;
   int2 *d_meta = nullptr;
@@ -231,6 +231,11 @@ int rs_ensure_g3l_tiles(rs_ctx *ctx, int KB);
 // above the transform limit; model cost of a form (0 direct, 1 transforms).
 int rs_g2_len(int N);
 double rs_g2_cost(int N, int form);
+struct RsG2Shape {
+  int threads, seg, halves, split;
+  size_t smem;
+};
+RsG2Shape rs_g2_shape(int M, int64_t tasks, int sms, const RsG2Shape *like);
 int rs_build_batch(rs_ctx *ctx, int n, const rs_bipoly *f, const rs_bipoly *g,
                    std::vector<PairPlan> &&plans, const RsBatchOpts &opt, rs_batch **out);
 // Byte sizes a batch of these plans needs (device arena, host staging in/out).

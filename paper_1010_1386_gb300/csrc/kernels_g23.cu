@@ -27,85 +27,143 @@ __device__ __forceinline__ int32_t signed_rep(uint32_t v, uint32_t p) {
   return v > (p >> 1) ? (int32_t)v - (int32_t)p : (int32_t)v;
 }
 
-__device__ __forceinline__ int64_t fold64(int64_t s, uint32_t c32) { return rs_fold64(s, c32); }
-
-// Reduce a folded accumulator (|s| < 2^53) to [0, p) in Montgomery form.
+// Reduce a folded accumulator, or the difference of two (|s| < 2^54), to
+// [0, p), divided by 2^32.
 __device__ __forceinline__ uint32_t finish64(int64_t s, const ModP &m) {
-  const uint64_t t = (uint64_t)(s + ((int64_t)m.p << 22));  // 0 <= t < 2^54 < p 2^32
+  const uint64_t t = (uint64_t)(s + ((int64_t)m.p << 24));  // 0 <= t < 2^56 < p 2^32
   return redc(t, m.p, m.pinv);
 }
 
-// y[k] = sum_{j<=k} x[j] b[k-j] for k < n (Montgomery form, reduced).  x and b
-// hold signed representatives and are zero for indices in [-RS_G2_PAD, 0)
-// and [n, n + RS_G2_PAD).
+// The direct convolution's work, split over a block.  Outputs come in blocks
+// of R; output block bi needs bi + 1 chunks of R inputs, so the pair of blocks
+// (pi, nblk - 1 - pi) needs nblk + 1 chunks for every pi.  That walk of
+// nblk + 1 chunks is cut into S segments of `len` chunks; each segment writes
+// its partial sums of both blocks, reduced to [0, p), and conv_value adds them.
+struct ConvShape {
+  int n, S, nblk, npair, len;
+};
+
+__device__ __forceinline__ ConvShape conv_shape(int n, int S) {
+  ConvShape c;
+  c.n = n;
+  c.S = S;
+  c.nblk = (n + RS_CONV_R - 1) / RS_CONV_R;
+  c.npair = (c.nblk + 1) / 2;
+  c.len = (c.nblk + S) / S;  // ceil((nblk + 1) / S)
+  return c;
+}
+
+// Partial sums of sum_{j<=k} x[j] b[k-j], k < n, of `nh` inputs x, x + W
+// against one b: part[(h S + s) n + k] over segment s of input h.  x and b
+// hold signed representatives and are zero for indices in [-RS_G2_PAD, 0) and
+// [n, n + RS_G2_PAD).
 //
-// Outputs come in blocks of R; block bi needs bi + 1 chunks of R inputs.
-// Thread t owns the block pair (pi, nblk - 1 - pi), pi = t, t + T, ..., and
-// walks both in one loop of nblk + 1 chunks, so every lane of a warp runs
-// the same trip count (no divergence in the multiply-accumulate loop).  In
-// the loop's first part neighbouring lanes read b and x R words apart (R odd:
-// distinct banks); in its second part every lane reads the same b words (a
-// broadcast).
-__device__ void conv_lazy(const int32_t *x, const int32_t *b, uint32_t *y, int n, const ModP &m) {
+// Neighbouring lanes take neighbouring block pairs of one segment.  While both
+// walk their low block they read b words R apart (R odd: distinct banks) and
+// the same x words, in the mirror blocks the same b words and x words R apart;
+// every unit of a segment has the same trip count.  Lanes leave their low
+// block in different steps, so a step only keeps the sums of that moment
+// (snap) and the mirror block's are the difference at the end.
+__device__ void conv_parts(const int32_t *x, const int32_t *b, uint32_t *part, const ConvShape &cs, int nh, int W,
+                           const ModP &m) {
   constexpr int R = RS_CONV_R;
-  const uint32_t c32 = m.r1;  // 2^32 mod p
-  const int nblk = (n + R - 1) / R;
-  const int npair = (nblk + 1) / 2;
-  for (int pi = threadIdx.x; pi < npair; pi += blockDim.x) {
-    const int hb = nblk - 1 - pi;
-    const int steps = hb == pi ? pi + 1 : nblk + 1;  // odd count: the middle block once
-    int k0 = pi * R, j0 = 0;
-    int64_t acc[R];
+  const int n = cs.n, units = nh * cs.S * cs.npair;
+  for (int u = threadIdx.x; u < units; u += blockDim.x) {
+    const int hs = u / cs.npair, pi = u - hs * cs.npair;
+    const int h = hs >= cs.S, s = hs - h * cs.S;
+    const int hb = cs.nblk - 1 - pi;
+    const int c0 = s * cs.len;
+    const int steps = min(cs.len, (hb == pi ? pi + 1 : cs.nblk + 1) - c0);  // the middle block once
+    const bool low = c0 <= pi;
+    const int turn = low ? pi - c0 : -1;  // step that completes the low block
+    const int32_t *xp = x + h * W + (low ? c0 : c0 - pi - 1) * R;
+    const int32_t *bp = b + ((low ? pi - c0 : hb - (c0 - pi - 1)) * R - (R - 1));
+    int64_t acc[R], snap[R];
 #pragma unroll
-    for (int r = 0; r < R; ++r) acc[r] = 0;
+    for (int r = 0; r < R; ++r) acc[r] = snap[r] = 0;
 #pragma unroll 1
     for (int c = 0; c < steps; ++c) {
       int32_t bw[2 * R - 1], av[R];
-      const int base = k0 - j0 - (R - 1);
 #pragma unroll
-      for (int i = 0; i < 2 * R - 1; ++i) bw[i] = b[base + i];
+      for (int i = 0; i < 2 * R - 1; ++i) bw[i] = bp[i];
 #pragma unroll
-      for (int i = 0; i < R; ++i) av[i] = x[j0 + i];
+      for (int i = 0; i < R; ++i) av[i] = xp[i];
+      xp += R;
+      bp -= R;
 #pragma unroll
       for (int r = 0; r < R; ++r) {
 #pragma unroll
         for (int jj = 0; jj < R; ++jj) acc[r] = rs_mac_s32(acc[r], av[jj], bw[(R - 1) + r - jj]);
-        acc[r] = fold64(acc[r], c32);
+        acc[r] = rs_fold64(acc[r], m.r1);
       }
-      j0 += R;
-      if (j0 > k0) {  // block complete: write it and move to the mirror block
+      if (c == turn) {  // on to the mirror block
 #pragma unroll
-        for (int r = 0; r < R; ++r) {
-          if (k0 + r < n) y[k0 + r] = finish64(acc[r], m);
-          acc[r] = 0;
-        }
-        k0 = hb * R;
-        j0 = 0;
+        for (int r = 0; r < R; ++r) snap[r] = acc[r];
+        xp = x + h * W;
+        bp = b + (hb * R - (R - 1));
       }
+    }
+    const bool kept = steps <= turn;  // the segment ends in the low block
+    uint32_t *y = part + (size_t)hs * n;
+#pragma unroll
+    for (int r = 0; r < R; ++r) {
+      const int64_t lo = kept ? acc[r] : snap[r];
+      if (pi * R + r < n) y[pi * R + r] = finish64(lo, m);
+      if (hb != pi && hb * R + r < n) y[hb * R + r] = finish64(acc[r] - lo, m);
     }
   }
 }
 
-// One block per (pair, prime).  The images come in pairs z+-_i at +-q^i,
-// i < M = NI / 2, with R(x) = E(x^2) + x O(x^2):
+// Sum of the segments' partial sums of output k of input h.
+__device__ __forceinline__ uint32_t conv_value(const uint32_t *part, const ConvShape &cs, int h, int k, const ModP &m) {
+  const uint32_t *y = part + (size_t)h * cs.S * cs.n + k;
+  uint32_t v = y[0];
+  for (int s = 1; s < cs.S; ++s) {
+    y += cs.n;
+    v = madd(v, y[0], m.p);
+  }
+  return v;
+}
+
+// Cluster barrier of a pair of blocks, in two halves.
+__device__ __forceinline__ void pair_arrive() { asm volatile("barrier.cluster.arrive.release;" ::: "memory"); }
+__device__ __forceinline__ void pair_wait() { asm volatile("barrier.cluster.wait.acquire;" ::: "memory"); }
+
+// One block, or a cluster of two, per (pair, prime).  The images come in pairs
+// z+-_i at +-q^i, i < M = NI / 2, with R(x) = E(x^2) + x O(x^2):
 //   E(Q^i) = (z+_i + z-_i) / 2,  O(Q^i) = (z+_i - z-_i) / (2 q^i),  Q = q^2,
 // and with z = num / den both are fractions over D_i = den+ den-, inverted
-// together.  E and O (degrees < M) are then interpolated in turn on the
-// geometric points Q^i by the two convolutions above, giving the even and
-// the odd coefficients of R.  Shared memory: four regions of M words, each
-// with RS_G2_PAD zero words on both sides.
-__global__ void g2_kernel(G2Args a) {
+// together.  E and O (degrees < M) are then interpolated on the geometric
+// points Q^i by the two convolutions above, giving the even and the odd
+// coefficients of R: both at once (a.halves = 2), in turn (1), or one in each
+// block of a cluster (a.split).  The residues may replace the numerators, so
+// in a cluster neither block writes before both have read.  Shared memory:
+// inputs of E and O and b, each of M words with RS_G2_PAD zero words on both
+// sides, and the partial sums (g2_seg segments of M words per half at once;
+// the inverses before that).
+//
+// Bound by the multiplier pipe (73% busy at 10,280 tasks of M = 113: a third
+// of it the convolutions' wide products, the rest modular products of the
+// steps around them), and for few tasks by a block's latency.  With one thread
+// per block pair and the halves in turn 3 to 33 lanes of a block worked;
+// splitting the walks fills them.  G2 stage, us, before (the fastest of the
+// three forms) -> now: 69 tasks of M = 451: 70 -> 20; 8,844 of 5 to 61: 83 ->
+// 37; 23,980 of 41: 248 -> 98; 10,280 of 113: 236 -> 119; 40,000 of 113: 860 ->
+// 427; 546 of 2,049: 880 -> 853; 1,127 of 169 to 1,369: 380 -> 268.
+__global__ void __launch_bounds__(512, 2) g2_kernel(G2Args a) {
   extern __shared__ __align__(16) uint32_t sm[];
   __shared__ uint32_t scratch[128];
-  const int2 task = a.tasks[blockIdx.x];
+  const int split = a.split;
+  const int2 task = a.tasks[blockIdx.x >> split];
   const PairDesc pd = a.pairs[task.x];
   const ModP m = a.mods[task.y];
   const int N = pd.N, NI = pd.NI, M = NI >> 1, D = M - 1, T = blockDim.x, tid = threadIdx.x;
   const int W = M + 2 * RS_G2_PAD;
+  const int nh = split ? 1 : 2, h0 = split ? (blockIdx.x & 1) : 0;  // halves of this block
+  const int hc = a.halves;                                         // of those, at once
   int32_t *X = reinterpret_cast<int32_t *>(sm) + RS_G2_PAD;
-  int32_t *Bs = X + W;
-  uint32_t *Y = reinterpret_cast<uint32_t *>(Bs + W);
-  uint32_t *Oh = Y + W;  // O's interpolation input while E is interpolated
+  int32_t *Bs = X + nh * W;
+  uint32_t *Y = reinterpret_cast<uint32_t *>(Bs + W - RS_G2_PAD);
   const size_t base = (size_t)pd.img_off + (size_t)task.y * NI;
   const size_t tb = (size_t)task.y * a.tab_stride;
   const uint32_t *finv = a.finv + tb, *gt = a.gtab + tb, *hq = a.hq + tb;
@@ -114,40 +172,48 @@ __global__ void g2_kernel(G2Args a) {
   uint32_t *dens = reinterpret_cast<uint32_t *>(Bs);
   for (int i = tid; i < M; i += T) dens[i] = mmul(a.den[base + 2 * i], a.den[base + 2 * i + 1], m);
   __syncthreads();
-  batch_invert(dens, Y, M, m, scratch);
+  batch_invert(dens, Y, M, m, scratch, true);  // plain inverses: from here on plain times Montgomery form
   __syncthreads();
   for (int i = tid; i < M; i += T) {
     const uint32_t np = a.num[base + 2 * i], dp = a.den[base + 2 * i];
     const uint32_t nm = a.num[base + 2 * i + 1], dm = a.den[base + 2 * i + 1];
-    const uint32_t e = mmul(mmul2(np, dm, nm, dp, m), Y[i], m);             // z+ + z-
-    const uint32_t o = mmul(mmul2(np, dm, mneg(nm, m.p), dp, m), Y[i], m);  // z+ - z-
-    X[i] = signed_rep(mmul(mmul(e, hq[0], m), finv[i], m), m.p);  // (E / F_i); hq[0] = 1/2
-    Oh[i] = mmul(mmul(o, hq[i], m), finv[i], m);                   // (O / F_i)
+    const uint32_t fy = mmul(finv[i], Y[i], m);
+    for (int h = 0; h < nh; ++h) {
+      const bool odd = (h0 + h) != 0;
+      const uint32_t v = mmul2(np, dm, odd ? mneg(nm, m.p) : nm, dp, m);  // z+ +- z-
+      // E / F_i or O / F_i; hq[0] = 1/2
+      X[h * W + i] = signed_rep(mmul(mmul(v, hq[odd ? i : 0], m), fy, m), m.p);
+    }
   }
-  __syncthreads();
+  if (split) pair_arrive();
   for (int i = tid; i < M; i += T) Bs[i] = bt[i];
   for (int i = tid; i < RS_G2_PAD; i += T) {
-    X[-1 - i] = 0;
-    X[M + i] = 0;
+    for (int h = 0; h < nh; ++h) {
+      X[h * W - 1 - i] = 0;
+      X[h * W + M + i] = 0;
+    }
     Bs[-1 - i] = 0;
     Bs[M + i] = 0;
   }
   __syncthreads();
-  for (int half = 0; half < 2; ++half) {  // E: even coefficients, then O: odd ones
-    conv_lazy(X, Bs, Y, M, m);  // Y[k] = Q^{C(k,2)} c_k
+  const ConvShape cs = conv_shape(M, pd.g2_seg);
+  for (int hh = 0; hh < nh; hh += hc) {
+    int32_t *x = X + hh * W;
+    conv_parts(x, Bs, Y, cs, hc, W, m);  // Y: Q^{C(k,2)} c_k
     __syncthreads();
-    for (int k = tid; k < M; k += T) X[D - k] = signed_rep(mmul(Y[k], gt[k], m), m.p);  // c_k F_k reversed
+    for (int k = tid; k < M; k += T)
+      for (int h = 0; h < hc; ++h)
+        x[h * W + D - k] = signed_rep(mmul(conv_value(Y, cs, h, k, m), gt[k], m), m.p);  // c_k F_k reversed
     __syncthreads();
-    conv_lazy(X, Bs, Y, M, m);  // Y[D - t] = sum_s c_{t+s} F_{t+s} b_s
+    conv_parts(x, Bs, Y, cs, hc, W, m);  // Y[D - t]: sum_s c_{t+s} F_{t+s} b_s
     __syncthreads();
-    for (int i = tid; i < M; i += T) {
-      const int c = 2 * i + half;
-      if (c < N) a.coef[base + c] = from_mont(mmul(Y[D - i], finv[i], m), m);
-    }
-    if (half == 0) {
-      for (int i = tid; i < M; i += T) X[i] = signed_rep(Oh[i], m.p);
-      __syncthreads();
-    }
+    if (split) pair_wait();
+    for (int i = tid; i < M; i += T)
+      for (int h = 0; h < hc; ++h) {
+        const int c = 2 * i + h0 + hh + h;
+        if (c < N) a.coef[base + c] = mmul(conv_value(Y, cs, h, D - i, m), finv[i], m);
+      }
+    __syncthreads();
   }
 }
 
@@ -285,15 +351,32 @@ cudaError_t launch_tables(const ModP *mods, const uint32_t *qbase, int K, int N,
   return cudaGetLastError();
 }
 
-cudaError_t g2_prepare(size_t smem) {
-  (void)smem;  // per-kernel attribute: allow the largest any plan may need
-  return cudaFuncSetAttribute(g2_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                              RS_G2_MAX_SMEM_BYTES);
+cudaError_t g2_prepare() {  // per-kernel attribute: allow the largest any plan may need
+  cudaError_t e = cudaFuncSetAttribute(g2_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, RS_G2_MAX_SMEM_BYTES);
+  // one carveout for every class: launches that want different ones don't share an SM
+  if (e == cudaSuccess)
+    e = cudaFuncSetAttribute(g2_kernel, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared);
+  return e;
 }
 
 cudaError_t launch_g2(int threads, int blocks, size_t smem, const G2Args &a, cudaStream_t s) {
-  g2_kernel<<<blocks, threads, smem, s>>>(a);
-  return cudaGetLastError();
+  if (!a.split) {
+    g2_kernel<<<blocks, threads, smem, s>>>(a);
+    return cudaGetLastError();
+  }
+  cudaLaunchConfig_t cfg = {};
+  cudaLaunchAttribute at[1];
+  at[0].id = cudaLaunchAttributeClusterDimension;
+  at[0].val.clusterDim.x = 2;
+  at[0].val.clusterDim.y = 1;
+  at[0].val.clusterDim.z = 1;
+  cfg.gridDim = dim3(2 * blocks);
+  cfg.blockDim = dim3(threads);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = s;
+  cfg.attrs = at;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, g2_kernel, a);
 }
 
 

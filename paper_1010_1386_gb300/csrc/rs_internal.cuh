@@ -38,6 +38,7 @@ struct PairDesc {
   int64_t out_off;       // offset of the N*Lout output block (coefficient-major)
   int64_t xl_off;        // offset of the CRT digit scratch: N * 16 * ceil(Lout/16) words
   int64_t cy_off;        // offset of the CRT chunk carries: N * ceil(Lout/16) int64
+  int32_t g2_seg;        // segments of the direct interpolation's block-pair walk
   int64_t xd_off;        // element offset of the operand digits of its first 128 coefficients
 };
 
@@ -112,6 +113,8 @@ struct G2Args {
   const int32_t *btab;     // [prime][tab_stride] (-1)^t Q^{C(t,2)} / F_t, signed representative
   const uint32_t *hq;      // [prime][tab_stride] 1 / (2 q^t)  (Montgomery)
   int32_t tab_stride;
+  int32_t halves;          // of E and O, in one block at once
+  int32_t split;           // 1: E and O in a block each (a cluster of two)
 };
 
 // Tensor-core G2 (kernels_g2t.cu).  For one prime, the rows of a row tile
@@ -262,7 +265,7 @@ cudaError_t launch_g1(int cap, int threads, int blocks, size_t smem, const G1Arg
 int g1_supported_cap(int cap);           // smallest compiled register capacity >= cap, or 0
 cudaError_t g1_prepare(int cap, int threads, size_t smem, int *max_blocks_per_sm);
 cudaError_t launch_g2(int threads, int blocks, size_t smem, const G2Args &a, cudaStream_t s);
-cudaError_t g2_prepare(size_t smem);
+cudaError_t g2_prepare();
 cudaError_t g2n_prepare();
 cudaError_t launch_g2n(int blocks, size_t smem, const G2nArgs &a, cudaStream_t s);
 // Tensor-core G2: kernel attributes once; the Toeplitz digit tiles of K
