@@ -951,6 +951,7 @@ int rs_build_batch(rs_ctx *ctx, int n, const rs_bipoly *f, const rs_bipoly *g,
   for (int i : order) {
     const PairPlan &p = b->plans[i];
     const int di = b->dev_index[i], chunks = (p.Lout + 15) / 16;
+    b->g3_maxL = std::max(b->g3_maxL, p.Lout);
     for (int j = 0; j < p.N; j += 128) g3.push_back(make_int2(di, j));
     for (int j = 0; j < p.N; j += b->g3_jt) g3d.push_back(make_int2(di, j));  // digit tiles
     for (int c = 0; c < chunks; ++c)
@@ -1517,7 +1518,7 @@ static int enqueue(rs_batch *b, bool capturing) {
       RS_CUDA(ctx, launch_g3l(b->ng3b, al, s));
     }
     // the output kernel; the limb chunks unless the tensor cores formed the limbs
-    RS_CUDA(ctx, launch_g3bc(b->g3_tlimbs ? 0 : b->ng3b, b->ng3, a3, b->d_g3, s));
+    RS_CUDA(ctx, launch_g3bc(b->g3_tlimbs ? 0 : b->ng3b, b->ng3, b->g3_maxL, ctx->sms, a3, b->d_g3, s));
   }
   if (timing) RS_CUDA(ctx, record(b->ev[3], s, capturing));
   return RS_OK;

@@ -170,6 +170,7 @@ struct rs_batch {
   int64_t status_off = 0; // word offset of the device status word (0 = every bounded wait completed)
   int ng2 = 0, ng3 = 0;
   int ng3d = 0, ng3b = 0, kmax = 0;  // CRT digit tiles, limb chunks, largest K
+  int g3_maxL = 0;                   // output limbs of the longest coefficients
   int g3_jt = 32;                    // coefficients per CRT digit tile (32 or 16)
   bool g3_perthread = false;         // CRT digits with one thread per coefficient
   bool g3_tensor = false;            // CRT digits on the tensor cores (kernels_g3m.cu)

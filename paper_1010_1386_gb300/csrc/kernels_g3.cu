@@ -538,6 +538,125 @@ __global__ void __launch_bounds__(128) g3c_kernel(G3Args a) {
   atomicMax(a.shape + 2 * task.x + 1, need);
 }
 
+// The same with the chunks of a coefficient in parallel, for few coefficients
+// of many limbs:
+// One thread per coefficient and chunk (lanes: 32 coefficients, so the loads
+// are whole lines; threadIdx.y: blockDim.y chunks at a time; threadIdx.z:
+// groups of 32 coefficients).  With the previous chunk's carry added, a chunk
+// is W + 2^512 e0, 0 <= W < 2^512, and what it passes on is
+//   f(e) = e0 + floor((W + e) / 2^512),  e in {-2, ..., 1} from the chunks below
+// (the whole chunk is above -2^512 - 2^48 and below 2^512 + 2^48).  f's four
+// values go to shared memory packed in a byte, every thread walks the bytes of
+// the chunks below its own, adds its e, and the limbs leave through shared
+// memory as runs of one coefficient (out is [coefficient][limb]).
+//
+// Bound by a few dependent latencies per step of blockDim.y chunks.  CRT stage,
+// us, with one thread walking a coefficient's chunks -> here: 40 blocks of 122
+// chunks 2,120 -> 2,036; 20 of 74 545 -> 489; 33 of 34 253 -> 225; 40 of 31
+// 254 -> 229; 8 of 5 32.2 -> 30.3; but 4,899 blocks of 2 to 5 1,480 -> 1,630,
+// 1,047 of one or two 34.4 -> 40.6, 512 of 33 1,790 -> 1,823 and one of one
+// 16 -> 18 (short runs, more threads per limb): taken for three chunks or
+// more and at most two blocks per SM.
+constexpr int kG3cWords = 4 * 32 * (4 * 16 + 1);  // coefficients x (16 chunks' limbs + 1), over all splits
+
+__global__ void __launch_bounds__(512) g3cp_kernel(G3Args a) {
+  __shared__ uint32_t T[kG3cWords];  // T[t (16 G + 1) + 16 g + w]: limb 16 (c0 + g) + w of coefficient t
+  __shared__ uint32_t fn[2][512];
+  __shared__ int top[3][128];  // per coefficient: negative?, codes of the last limb != 0 and != 0xffffffff
+  const int2 task = a.tasks[blockIdx.x];
+  const PairDesc pd = a.pairs[task.x];
+  const int G = (int)blockDim.y, lane = (int)threadIdx.x, g = (int)threadIdx.y;
+  const int ct = (int)threadIdx.z * 32 + lane;  // coefficient of the block
+  const int j0 = task.y + (int)(blockIdx.y * blockDim.z) * 32, j = j0 + ct;
+  if (j0 >= pd.N) return;  // the whole block
+  const bool live = j < pd.N;
+  const int N = pd.N, L = pd.Lout, C = (L + 15) / 16, stride = 16 * G + 1;
+  const uint32_t *xl = a.xl + pd.xl_off + j;
+  const int64_t *cyp = a.carry + pd.cy_off + j;
+  const int p0 = __ldg(a.poff + pd.K);
+  const uint32_t *PK = reinterpret_cast<const uint32_t *>(a.p16 + p0);  // P's 32-bit limbs
+  // limbs from the signed digits (tensor-core limb kernel) need no offset: P = 0 here
+  const int plen = a.signed_digits ? 0 : (__ldg(a.poff + pd.K + 1) - p0) / 2;
+  uint32_t *o = a.out + pd.out_off;
+  if (g == 0) top[0][ct] = top[1][ct] = top[2][ct] = 0;
+  __syncthreads();
+  int e = 0;  // carry into the chunks of this step (equal for the threads of a coefficient)
+  for (int c0 = 0; c0 < C; c0 += G) {
+    const int c = c0 + g;
+    const bool act = live && c < C;
+    uint32_t x[16];
+    uint32_t f = 0xe4u;  // the identity: f(e) = e
+    if (act) {
+      int64_t r = c ? cyp[(size_t)(c - 1) * N] : 0;
+      uint32_t any = 0u, all = 0xffffffffu, rest = 0u, pk = 16 * c < plen ? __ldg(PK + 16 * c) : 0u;
+#pragma unroll
+      for (int w = 0; w < 16; ++w) x[w] = xl[(size_t)(16 * c + w) * N];
+#pragma unroll
+      for (int w = 0; w < 16; ++w) {
+        const uint32_t pn = 16 * c + w + 1 < plen ? __ldg(PK + 16 * c + w + 1) : 0u;
+        const uint32_t h = (pk >> 1) | (pn << 31);
+        pk = pn;
+        const int64_t v = (int64_t)x[w] + r - (int64_t)h;
+        x[w] = (uint32_t)v;
+        r = v >> 32;
+        any |= x[w];
+        all &= x[w];
+        if (w) rest |= x[w];
+      }
+      const int e0 = (int)r + 2;
+      f = (uint32_t)(e0 - (rest == 0u && x[0] < 2u ? 1 : 0)) | (uint32_t)(e0 - (any == 0u ? 1 : 0)) << 2 |
+          (uint32_t)e0 << 4 | (uint32_t)(e0 + (all == 0xffffffffu ? 1 : 0)) << 6;
+    }
+    uint32_t *fs = fn[(c0 / G) & 1];
+    fs[g * 32 * blockDim.z + ct] = f;
+    __syncthreads();
+    int mine = e;
+    for (int i = 0; i < G; ++i) {
+      if (i == g) mine = e;
+      e = (int)((fs[i * 32 * blockDim.z + ct] >> (2 * (e + 2))) & 3u) - 2;
+    }
+    if (act) {
+      int64_t r = mine;
+      int nz = 0, nf = 0;  // 2 (index + 1) + whether the sign needs one more limb
+#pragma unroll
+      for (int w = 0; w < 16; ++w) {
+        const int l = 16 * c + w;
+        const int64_t v = (int64_t)x[w] + r;
+        const uint32_t limb = (uint32_t)v;
+        r = v >> 32;
+        T[ct * stride + 16 * g + w] = limb;
+        if (l < L) {
+          if (limb != 0u) nz = 2 * (l + 1) + (int)(limb >> 31);
+          if (limb != 0xffffffffu) nf = 2 * (l + 1) + (int)(~limb >> 31);
+          if (l == L - 1) top[0][ct] = (int)(limb >> 31);
+        }
+      }
+      atomicMax(&top[1][ct], nz);
+      atomicMax(&top[2][ct], nf);
+    }
+    __syncthreads();
+    const int nl = min(16 * G, L - 16 * c0);  // limbs of this step that exist
+    for (int t = g; t < 32; t += G) {
+      const int tt = (int)threadIdx.z * 32 + t;
+      if (j0 + tt < N)
+        for (int w = lane; w < nl; w += 32) o[(size_t)(j0 + tt) * L + 16 * c0 + w] = T[tt * stride + w];
+    }
+  }
+  __syncthreads();
+  if (g != 0) return;
+  // fewest limbs whose two's-complement value is this coefficient
+  const bool neg = top[0][ct] != 0;
+  const int code = top[neg ? 2 : 1][ct];
+  const bool zero = !live || (!neg && code == 0);
+  const int need = zero ? 0 : max(1, min((code >> 1) + (code & 1), L));
+  const int len = __reduce_max_sync(0xffffffffu, zero ? 0 : j + 1);
+  const int most = __reduce_max_sync(0xffffffffu, need);
+  if (lane == 0 && len) {
+    atomicMax(a.shape + 2 * task.x, len);
+    atomicMax(a.shape + 2 * task.x + 1, most);
+  }
+}
+
 // W[k][l] = p_0 ... p_{l-1} mod p_k (Montgomery form, signed), one thread per k.
 __global__ void crt_w_kernel(const ModP *mods, int K, int32_t *wtab) {
   const int k = blockIdx.x * blockDim.x + threadIdx.x;
@@ -621,13 +740,20 @@ cudaError_t launch_g3p(int nt, const G3Args &a, const int2 *tasks, cudaStream_t 
   return cudaGetLastError();
 }
 
-cudaError_t launch_g3bc(int nb, int nc, const G3Args &a, const int2 *otasks, cudaStream_t s) {
+cudaError_t launch_g3bc(int nb, int nc, int maxL, int sms, const G3Args &a, const int2 *otasks, cudaStream_t s) {
   if (nb) g3b_kernel<<<nb, 128, 0, s>>>(a);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
   G3Args ao = a;
   ao.tasks = otasks;
-  if (nc) g3c_kernel<<<nc, 128, 0, s>>>(ao);
+  // Chunks in parallel: 16 (chunk, 32 coefficients) groups a block, as many
+  // chunks at once as the longest coefficient has, the 128 coefficients of a
+  // task in 1, 2 or 4 parts.
+  const int C = (maxL + 15) / 16, G = std::max(1, std::min(16, C)), Z = G <= 4 ? 4 : G <= 8 ? 2 : 1;
+  if (nc && C >= 3 && nc <= 2 * sms)
+    g3cp_kernel<<<dim3(nc, 4 / Z), dim3(32, G, Z), 0, s>>>(ao);
+  else if (nc)
+    g3c_kernel<<<nc, 128, 0, s>>>(ao);
   return cudaGetLastError();
 }
 

@@ -308,7 +308,7 @@ cudaError_t launch_yun(int ntasks, const YunArgs &a, cudaStream_t s);
 cudaError_t launch_g1s(int slots, int ntiles, size_t smem, const G1sArgs &a, cudaStream_t s);
 cudaError_t launch_g1s_fallback(int blocks, size_t smem, const G1sArgs &a, cudaStream_t s);
 cudaError_t launch_g2s(int ntasks, size_t smem, const G2sArgs &a, cudaStream_t s);
-cudaError_t launch_g3bc(int nb, int nc, const G3Args &a, const int2 *otasks, cudaStream_t s);
+cudaError_t launch_g3bc(int nb, int nc, int maxL, int sms, const G3Args &a, const int2 *otasks, cudaStream_t s);
 // Residues of one lifted factor divided by an integer g, prime by prime:
 // out[dst_off + k n + j] = in[src_off + k src_stride + j] * (g mod p_k)^{-1}
 // mod p_k for k < this factor's primes, j < n; g's 32-bit limbs (least

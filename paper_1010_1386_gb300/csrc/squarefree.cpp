@@ -705,10 +705,12 @@ extern "C" int rs_squarefree_batch(rs_ctx *ctx, int32_t n, const rs_bipoly *f, c
     const uint32_t one = 1u;
     std::vector<int2> g3d, g3;
     std::vector<int4> g3b;
+    int maxL = 0;
     for (int fi = 0; fi < nf; ++fi) {
       const PairDesc &pd = descs[fi];
       for (int j = 0; j < pd.N; j += 32) g3d.push_back(make_int2(fi, j));
       for (int j = 0; j < pd.N; j += 128) g3.push_back(make_int2(fi, j));
+      maxL = std::max(maxL, pd.Lout);
       for (int c = 0; c < (pd.Lout + 15) / 16; ++c)
         for (int j = 0; j < pd.N; j += 128) g3b.push_back(make_int4(fi, j, c, 0));
     }
@@ -783,7 +785,7 @@ extern "C" int rs_squarefree_batch(rs_ctx *ctx, int32_t n, const rs_bipoly *f, c
         e = cudaEventRecord(lev[0], s);
         if (e == cudaSuccess) e = launch_scale(d_gat, nf, kmax, ctx->d_mods, d_one, b->d_yun_out, d_qA, s);
         if (e == cudaSuccess) e = launch_g3t((int)g3d.size(), a3, d_g3d, s);
-        if (e == cudaSuccess) e = launch_g3bc((int)g3b.size(), (int)g3.size(), a3, d_g3, s);
+        if (e == cudaSuccess) e = launch_g3bc((int)g3b.size(), (int)g3.size(), maxL, ctx->sms, a3, d_g3, s);
         if (e == cudaSuccess) e = cudaEventRecord(lev[1], s);
       }
       const auto tf = std::chrono::steady_clock::now();
@@ -874,10 +876,12 @@ extern "C" int rs_squarefree_batch(rs_ctx *ctx, int32_t n, const rs_bipoly *f, c
     if (gw.empty()) gw.push_back(0u);
     std::vector<int2> g3dB, g3B;
     std::vector<int4> g3bB;
+    int maxLB = 0;
     for (int fi = 0; fi < nf; ++fi) {
       const PairDesc &q = dB[fi];
       for (int j = 0; j < q.N; j += 32) g3dB.push_back(make_int2(fi, j));
       for (int j = 0; j < q.N; j += 128) g3B.push_back(make_int2(fi, j));
+      maxLB = std::max(maxLB, q.Lout);
       for (int c = 0; c < (q.Lout + 15) / 16; ++c)
         for (int j = 0; j < q.N; j += 128) g3bB.push_back(make_int4(fi, j, c, 0));
     }
@@ -954,7 +958,7 @@ extern "C" int rs_squarefree_batch(rs_ctx *ctx, int32_t n, const rs_bipoly *f, c
         a3.shape = reinterpret_cast<int32_t *>(d_outB + outB);
         a3.kmax = kmaxB;
         e = launch_g3t((int)g3dB.size(), a3, d_g3d, s);
-        if (e == cudaSuccess) e = launch_g3bc((int)g3bB.size(), (int)g3B.size(), a3, d_g3, s);
+        if (e == cudaSuccess) e = launch_g3bc((int)g3bB.size(), (int)g3B.size(), maxLB, ctx->sms, a3, d_g3, s);
       }
       if (e == cudaSuccess) e = cudaEventRecord(qev[1], s);
       if (e == cudaSuccess)
