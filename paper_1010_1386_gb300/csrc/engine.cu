@@ -898,16 +898,22 @@ int rs_build_batch(rs_ctx *ctx, int n, const rs_bipoly *f, const rs_bipoly *g,
   // Digits: one thread per coefficient when there are enough of them for one
   // each to fill the GPU, the fewer the primes (a thread walks its K^2 / 2
   // products alone): from 96 per SM, 8 K per SM, 1024 per SM for any K.
-  // Otherwise tiles of 32 or 16 coefficients on the CUDA cores, or the tensor
-  // cores in tiles of 128, whichever these times (ms, fitted to the
-  // measurements below; 608 schedulers' products against one tile's chain of
-  // digit blocks per wave) say.  Limbs: on the tensor cores unless the digits
-  // took one thread per coefficient or no pair has 24 primes.
+  // Otherwise tiles of 32 or 16 coefficients on the CUDA cores, the tensor
+  // cores in tiles of 128, or, above 256 primes, two levels: tiles for 256
+  // digits at a time and their products with the later residues on the tensor
+  // cores of all SMs; whichever these times (ms, fitted to the measurements
+  // below; 608 schedulers' products against one tile's chain of digit blocks
+  // per wave, and for two levels both a group's chain and its waves of far
+  // products) say.  Limbs: on the tensor cores unless the digits took one
+  // thread per coefficient or no pair has 24 primes.
   // CRT stage, us: CUDA-core tiles with CUDA-core limbs, with tensor-core
   // limbs, tensor-core digits and limbs, one thread per coefficient (with the
   // digits' earlier kernel, which took one warp through each digit block's 64
   // steps, the first column was 79, 727, 694, 1,650 and 5,910 us in rows 3, 6,
   // 8, 10 and 11):
+  // Two levels, against the fastest of the others with the carry kernel of
+  // kernels_g3.cu: 4,097 of 546 229 -> 184, 4,520 of 514 232 -> 190, 1,640 of
+  // 1,199 504 -> 307, 4,520 of 2,000 2,028 -> 1,003, 63,008 of 526 1,792 -> 1,772.
   //   coefficients  primes (avg)  tiles  + limbs  tensor  per thread
   //     1,160         27             24      22      43      41
   //     3,178          8             24      24      43      30
@@ -942,11 +948,25 @@ int rs_build_batch(rs_ctx *ctx, int n, const rs_bipoly *f, const rs_bipoly *g,
     const int64_t sms = ctx->sms;
     b->g3_jt = nt32 < 2 * sms ? 16 : 32;
     b->g3_perthread = ncoef >= sms * std::min<int64_t>(RS_G3P_MIN_COEF_PER_SM, std::max(96, 8 * kc));
-    const double ms_tiles = std::max(1.1e-10 * nk2 * 152 / sms, 2.7e-7 * kc * kc);
+    const double ms_tiles = std::max(1.1e-10 * nk2 * 152 / sms + 0.6e-4 * kc, 2.7e-7 * kc * kc);
     const double ms_tensor = (double)((nt128 + sms - 1) / sms) * kc * 0.55e-3 * (1.0 + kc / 2500.0);
+    double ms_two = (kc / 256.0) * std::max(0.037, 0.008 + 0.022 / 16.0 * ncoef / sms);
+    for (int c = 4; 64 * c < kc; c += 4) {
+      int64_t items = 0;
+      for (int i : order) {
+        const int kb = (b->descs[b->dev_index[i]].K + 63) / 64;
+        if (kb > c) items += (int64_t)((b->plans[i].N + 127) / 128) * (kb - c);
+      }
+      ms_two += 0.004 + 0.009 * ((items + sms - 1) / sms);
+      ++b->g3_nfar;
+    }
     const bool tc = !b->g3_perthread && !images_only && ctx->cfg.crt_form != 1;
-    b->g3_tensor = tc && (ctx->cfg.crt_form == 2 || (kc >= RS_G3M_MIN_K && ms_tensor < ms_tiles));
-    b->g3_tlimbs = tc && (b->g3_tensor || kc >= RS_G3L_MIN_K);
+    b->g3_two = tc && ctx->cfg.crt_form != 2 && b->g3_nfar > 0 && ms_two < ms_tiles &&
+                (kc < RS_G3M_MIN_K || ms_two < ms_tensor);
+    if (!b->g3_two) b->g3_nfar = 0;
+    b->g3_tensor =
+        tc && !b->g3_two && (ctx->cfg.crt_form == 2 || (kc >= RS_G3M_MIN_K && ms_tensor < ms_tiles));
+    b->g3_tlimbs = tc && (b->g3_tensor || b->g3_two || kc >= RS_G3L_MIN_K);
   }
   for (int i : order) {
     const PairPlan &p = b->plans[i];
@@ -991,6 +1011,7 @@ int rs_build_batch(rs_ctx *ctx, int n, const rs_bipoly *f, const rs_bipoly *g,
                             (b->nyun > 0) +
                             (b->ng3b > 0) +
                             (b->ng3 > 0);
+  b->info.kernel_launches += b->g3_two ? b->g3_nfar + ((maxK + 63) / 64 + 3) / 4 - 1 : 0;
   for (const auto &gc : b->g2cls)
     if (gc.tensor) b->info.kernel_launches += 4;  // five launches per tensor-core class
 
@@ -999,7 +1020,7 @@ int rs_build_batch(rs_ctx *ctx, int n, const rs_bipoly *f, const rs_bipoly *g,
   for (int lg = 1; lg <= RS_NTT_LGMAX && rc == RS_OK; ++lg)
     if (bhatK[lg]) rc = rs_ensure_bhat(ctx, lg, bhatK[lg]);
   if (rc == RS_OK && g2t_kmax > 0) rc = rs_ensure_g2t_btile(ctx, g2t_kmax, g2t_tiles);
-  if (rc == RS_OK && b->g3_tensor) rc = rs_ensure_g3m_wtiles(ctx, (maxK + 63) / 64);
+  if (rc == RS_OK && (b->g3_tensor || b->g3_two)) rc = rs_ensure_g3m_wtiles(ctx, (maxK + 63) / 64);
   if (rc == RS_OK && b->g3_tlimbs) rc = rs_ensure_g3l_tiles(ctx, (maxK + 63) / 64);
   if (rc == RS_OK && b->g3_tlimbs) {
     // The limbs then come from the tensor cores too: one task per (digit
@@ -1156,7 +1177,7 @@ int rs_build_batch(rs_ctx *ctx, int n, const rs_bipoly *f, const rs_bipoly *g,
       if (e2 != cudaSuccess) rc = rs_fail(ctx, RS_ERR_CUDA, std::string("G2 set-up: ") + cudaGetErrorString(e2));
       ctx->g2n_ready = e2 == cudaSuccess;
     }
-    if (rc == RS_OK && b->g3_tensor && !ctx->g3m_ready) {
+    if (rc == RS_OK && (b->g3_tensor || b->g3_two) && !ctx->g3m_ready) {
       cudaError_t e2 = g3m_prepare();
       if (e2 != cudaSuccess) rc = rs_fail(ctx, RS_ERR_CUDA, std::string("G3 set-up: ") + cudaGetErrorString(e2));
       ctx->g3m_ready = e2 == cudaSuccess;
@@ -1496,6 +1517,32 @@ static int enqueue(rs_batch *b, bool capturing) {
       am.err = reinterpret_cast<int32_t *>(b->d_out + b->status_off);
       am.stall = ctx->d_stall;
       RS_CUDA(ctx, launch_g3m(b->ng3, am, s));
+    } else if (b->g3_two) {
+      // groups of four digit blocks: their digits, then their products with the rest
+      G3uArgs au;
+      au.pairs = b->d_pairs;
+      au.tasks = b->d_g3;
+      au.mods = ctx->d_mods;
+      {
+        std::lock_guard<std::mutex> lock(ctx->tab_mu);
+        au.wtiles = ctx->g3m_wt;
+      }
+      au.coef = b->d_num;
+      au.xdig = b->d_g3m_x;
+      au.xoff = b->d_g3m_xoff;
+      au.ntasks = b->ng3;
+      au.err = reinterpret_cast<int32_t *>(b->d_out + b->status_off);
+      au.stall = ctx->d_stall;
+      const int KB = (b->kmax + 63) / 64;
+      for (int c = 0; c < KB; c += 4) {
+        a3.kbeg = 64 * c;
+        a3.kend = 64 * (c + 4);
+        RS_CUDA(ctx, launch_g3t(b->ng3d, a3, b->d_g3d, s, b->g3_jt));
+        au.c0 = c;
+        au.c1 = c + 4;
+        au.nkb = KB - au.c1;
+        if (au.nkb > 0) RS_CUDA(ctx, launch_g3u(ctx->sms, au, s));
+      }
     } else {
       RS_CUDA(ctx, launch_g3t(b->ng3d, a3, b->d_g3d, s, b->g3_jt));
     }

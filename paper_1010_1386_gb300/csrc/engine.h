@@ -174,6 +174,8 @@ struct rs_batch {
   int g3_jt = 32;                    // coefficients per CRT digit tile (32 or 16)
   bool g3_perthread = false;         // CRT digits with one thread per coefficient
   bool g3_tensor = false;            // CRT digits on the tensor cores (kernels_g3m.cu)
+  bool g3_two = false;               // CRT digits in two levels: tiles near, tensor cores far (g3u_kernel)
+  int g3_nfar = 0;                   // launches of its far products
   bool g3_tlimbs = false;            // CRT limbs on the tensor cores (kernels_g3l.cu)
   int64_t g3m_x_elems = 0;           // their operand digits
   uint16_t *d_g3m_x = nullptr;

@@ -98,7 +98,8 @@ __global__ void __launch_bounds__(128 * LS, 4 / LS) g3t_kernel(G3Args a) {
   const int rg = ltid >> 4, cg = ltid & 15;  // rows 8 rg .. 8 rg + 7, columns CJ cg .. CJ cg + CJ - 1
   uint32_t *col = a.coef + pd.img_off;       // residue, then digit, of (k, j) at col[k S + j]
   auto group_sync = [&] { asm volatile("bar.sync %0, 128;" ::"r"(grp + 1) : "memory"); };
-  for (int k0 = 0; k0 < K; k0 += G3T_BK) {
+  const int kend = a.kend ? min(K, a.kend) : K;
+  for (int k0 = a.kbeg; k0 < kend; k0 += G3T_BK) {
     const int bk = min(G3T_BK, K - k0);
     // Chunks of W (16 rows of one column per thread) and digits are loaded into
     // registers one chunk ahead, so their latency overlaps the products.
@@ -115,8 +116,8 @@ __global__ void __launch_bounds__(128 * LS, 4 / LS) g3t_kernel(G3Args a) {
 #pragma unroll
       for (int q = 0; q < NV; ++q) vreg[q] = vlive ? (int32_t)vcol[(size_t)(l0 + q * (128 / JT)) * S] : 0;
     };
-    const int nch = k0 / G3T_LC;  // k0 is a multiple of G3T_LC: full chunks
-    if (grp < nch) fetch(grp * G3T_LC);
+    const int nch = (k0 - a.kbeg) / G3T_LC;  // k0 and kbeg are multiples of 64: full chunks
+    if (grp < nch) fetch(a.kbeg + grp * G3T_LC);
     const int32_t *tri = a.wtri + (size_t)(k0 / G3T_BK) * (G3T_BK * G3T_BK);
 #pragma unroll
     for (int e = tid; e < G3T_BK * G3T_BK / 4; e += 128 * LS) {  // piece (s, r): not all zero, and used
@@ -143,7 +144,7 @@ __global__ void __launch_bounds__(128 * LS, 4 / LS) g3t_kernel(G3Args a) {
 #pragma unroll
       for (int q = 0; q < NV; ++q) Vs[grp][(ltid + 128 * q) / JT][ltid % JT] = vreg[q];
       group_sync();
-      if (ch + LS < nch) fetch((ch + LS) * G3T_LC);
+      if (ch + LS < nch) fetch(a.kbeg + (ch + LS) * G3T_LC);
       if (16 * warp < bk) {
 #pragma unroll 1
         for (int c0 = 0; c0 < G3T_LC; c0 += 8) {

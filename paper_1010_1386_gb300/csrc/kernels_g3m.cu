@@ -105,6 +105,20 @@ __device__ __forceinline__ void tmem_hold8(uint32_t *v) {
                : "+r"(v[0]), "+r"(v[1]), "+r"(v[2]), "+r"(v[3]), "+r"(v[4]), "+r"(v[5]), "+r"(v[6]), "+r"(v[7])::"memory");
 }
 
+// Column t of one window's seven classes: each an exact integer below 13.5 2^20
+// (at most 4.5 chunks of 64 inputs), taken by cvt.rni and combined with its
+// weight 256^s (2^32 = r1 <= 2^21, 2^48 = w48 mod p) into one int64 term below
+// 2^52.3, reduced by REDC.
+__device__ __forceinline__ uint32_t window_value(const uint32_t (&v)[7][8], int t, const ColConst &cq) {
+  int32_t c[7];
+#pragma unroll
+  for (int k = 0; k < 7; ++k) c[k] = __float2int_rn(__uint_as_float(v[k][t]));
+  const int64_t lo = (int64_t)c[0] + (int64_t)c[1] * 256 + (int64_t)c[2] * 65536 + (int64_t)c[3] * 16777216;
+  const int64_t mid = (int64_t)c[4] + (int64_t)c[5] * 256;
+  const int64_t x = lo + mid * (int64_t)cq.r1 + (int64_t)c[6] * (int64_t)cq.w48;
+  return finish64_t(x, mod_of(cq));
+}
+
 // Read-out windows of block kb: ceil(kb / kWin) over its earlier chunks; half
 // 1 also takes the products of the block's first 32 digits (its "rect"),
 // appended to its last window (alone when kb = 0), when the block has primes
@@ -359,11 +373,7 @@ __global__ void __launch_bounds__(kThreads, 1) g3m_kernel(G3mArgs a) {
         tc_fence_before();
       }
       auto readout = [&](const int hh) {
-        // One window of half hh's accumulator: each class an exact integer
-        // below 13.5 2^20 (at most 4.5 chunks of 64 inputs), taken by
-        // cvt.rni and combined with its weight 256^s (2^32 = r1 <= 2^21,
-        // 2^48 = w48 mod p) into one int64 term below 2^52.3, reduced at
-        // once (REDC, as every window's) and added mod p.
+        // One window of half hh's accumulator, added mod p.
         ok = ok && mbar_wait(b_accfull + 8 * hh, (hh ? rc1 : rc0) & 1, &abort_flag, a.err);
         if (hh)
           ++rc1;
@@ -393,14 +403,7 @@ __global__ void __launch_bounds__(kThreads, 1) g3m_kernel(G3mArgs a) {
 #pragma unroll
           for (int t = 0; t < 8; ++t) {
             const ColConst &cq = (hh ? c1 : cc0)[8 * grp + t];
-            int32_t c[7];
-#pragma unroll
-            for (int k = 0; k < 7; ++k) c[k] = __float2int_rn(__uint_as_float(v[k][t]));
-            const int64_t lo = (int64_t)c[0] + (int64_t)c[1] * 256 + (int64_t)c[2] * 65536 +
-                               (int64_t)c[3] * 16777216;
-            const int64_t mid = (int64_t)c[4] + (int64_t)c[5] * 256;
-            const int64_t x = lo + mid * (int64_t)cq.r1 + (int64_t)c[6] * (int64_t)cq.w48;
-            const uint32_t val = finish64_t(x, mod_of(cq));
+            const uint32_t val = window_value(v, t, cq);
             if (hh)
               s8[t] = madd(s8[t], val, cq.p);
             else
@@ -506,6 +509,186 @@ __global__ void __launch_bounds__(kThreads, 1) g3m_kernel(G3mArgs a) {
   }
 }
 
+// The far products of the two-level digits: the digits of chunks [c0, c1)
+// (at most kWin, one read-out window), which the tiled kernel of kernels_g3.cu
+// has written as operand digits, taken out of the residues of every later digit
+// block,
+//   r_k -= sum_{64 c0 <= l < 64 c1} v_l W[k][l]  mod p_k,  k >= 64 c1.
+// Items are (task, digit block kb >= c1), the tasks of one kb next to each
+// other (they share its W tiles in L2); a persistent block takes every
+// gridDim.x-th.  Products and read-out as in g3m_kernel, both halves at once:
+// warps 0-3 read out half 0, warps 4-7 half 1, and the next item's first two
+// chunks are copied meanwhile.
+//
+// Bound by the copies (96 KB per 64 digits from L2 for 128 coefficients and 64
+// primes) and the read-out, about 5 us an item; what it buys is that all SMs
+// share the products, where a block of g3m_kernel walks a tile's alone.
+// Measured: see the choice of the digit kernels in engine.cu.
+__global__ void __launch_bounds__(kThreads, 1) g3u_kernel(G3uArgs a) {
+  extern __shared__ __align__(1024) uint8_t sm[];
+  __shared__ __align__(8) uint64_t bar[7];  // full[2], empty[2], accfull, accfree, drain
+  __shared__ uint32_t tmem_slot;
+  __shared__ volatile int abort_flag;
+  __shared__ ColConst cc[kBlkK];
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const uint32_t sbase = smem_u32(sm);
+  const uint32_t b_full = smem_u32(&bar[0]), b_empty = smem_u32(&bar[2]);
+  const uint32_t b_accfull = smem_u32(&bar[4]), b_accfree = smem_u32(&bar[5]), b_drain = smem_u32(&bar[6]);
+  if (threadIdx.x == 0) {
+    abort_flag = 0;
+    for (int i = 0; i < 2; ++i) {
+      mbar_init(b_full + 8 * i, 1);
+      mbar_init(b_empty + 8 * i, 1);
+    }
+    mbar_init(b_accfull, 1);
+    mbar_init(b_accfree, 8);  // one arrival per read-out warp
+    mbar_init(b_drain, 1);
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+  }
+  if (warp == 8) {
+    asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], 512;" ::"r"(smem_u32(&tmem_slot))
+                 : "memory");
+    asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
+  }
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  const uint32_t tbase = tmem_slot;
+  const int items = a.ntasks * a.nkb;
+  // pair and digit block of an item; false when the pair has no such block
+  auto item_of = [&](int it, int &t, int &kb) {
+    kb = a.c1 + it / a.ntasks;
+    t = it % a.ntasks;
+    return kBlkK * kb < a.pairs[a.tasks[t].x].K;
+  };
+  if (warp == 9 && lane == 0) {  // producer
+    int g = 0;
+    bool ok = *a.stall == 0;  // test hook: no copies, so every consumer's wait runs out
+    for (int it = blockIdx.x; it < items && ok; it += gridDim.x) {
+      int t, kb;
+      if (!item_of(it, t, kb)) continue;
+      const uint8_t *xa = reinterpret_cast<const uint8_t *>(a.xdig + a.xoff[t]);
+      const uint8_t *wt = reinterpret_cast<const uint8_t *>(a.wtiles) + (size_t)(kb * (kb - 1) / 2) * 2 * kBStage;
+      for (int c = a.c0; c < a.c1; ++c, ++g) {
+        const int buf = g & 1;
+        if (g >= 2 && !mbar_wait(b_empty + 8 * buf, ((g - 2) >> 1) & 1, &abort_flag, a.err)) {
+          ok = false;
+          break;
+        }
+        const uint32_t dst = sbase + buf * kBuf, fb = b_full + 8 * buf;
+        mbar_expect_tx(fb, kBuf);
+        bulk_load(dst, xa + (size_t)c * kAChunk, kAChunk, fb);
+        bulk_load(dst + kAChunk, wt + (size_t)c * 2 * kBStage, 2 * kBStage, fb);
+      }
+    }
+    for (int q = g > 2 ? g - 2 : 0; q < g; ++q)
+      mbar_wait(b_full + 8 * (q & 1), (q >> 1) & 1, &abort_flag, a.err, false);
+  } else if (warp == 8 && lane == 0) {  // MMA issuer
+    int g = 0, n = 0;
+    bool ok = true;
+    for (int it = blockIdx.x; it < items && ok; it += gridDim.x) {
+      int t, kb;
+      if (!item_of(it, t, kb)) continue;
+      for (int c = a.c0; c < a.c1; ++c, ++g) {
+        const int buf = g & 1;
+        const bool first = c == a.c0;
+        if (!mbar_wait(b_full + 8 * buf, (g >> 1) & 1, &abort_flag, a.err) ||
+            (first && !mbar_wait(b_accfree, n & 1, &abort_flag, a.err))) {
+          ok = false;
+          break;
+        }
+        tc_fence_after();
+        const uint32_t abase = sbase + buf * kBuf, bbase = abase + kAChunk;
+#pragma unroll
+        for (int h = 0; h < 2; ++h)
+#pragma unroll
+          for (int u = 0; u < 2; ++u)
+#pragma unroll
+            for (int ks = 0; ks < 2; ++ks)
+#pragma unroll
+              for (int i = 0; i < 4; ++i)
+                tc_mma(tbase + h * kHalfCols + i * kHalf, sdesc(abase + u * kAStage + i * 8192 + ks * 256),
+                       sdesc(bbase + u * kBStage + h * kBHalf + ks * 256), !first || (u | ks | i) != 0);
+        tc_commit(b_empty + 8 * buf);
+      }
+      if (!ok) break;
+      tc_commit(b_accfull);
+      ++n;
+    }
+    tc_commit(b_drain);
+    mbar_wait(b_drain, 0, &abort_flag, a.err, false);
+  } else if (warp < 8) {
+    const int h = warp >> 2, q = warp & 3, row = 32 * q + lane;
+    const uint32_t tl = tbase + ((uint32_t)(32 * q) << 16) + h * kHalfCols;
+#pragma unroll
+    for (int z = 0; z < 3; ++z) tmem_zero32(tl + 128 + 32 * z);
+    tmem_wait_st();
+    tc_fence_before();
+    __syncwarp();
+    if (lane == 0) mbar_arrive(b_accfree);
+    int n = 0;
+    bool ok = true;
+    for (int it = blockIdx.x; it < items; it += gridDim.x) {
+      int t, kb;
+      if (!item_of(it, t, kb)) continue;
+      const int2 task = a.tasks[t];
+      const PairDesc &pd = a.pairs[task.x];
+      const int k0 = kBlkK * kb + kHalf * h, bk = min(kHalf, pd.K - k0), j = task.y + row, S = pd.NI;
+      uint32_t *col = a.coef + pd.img_off + (size_t)k0 * S + j;
+      const bool live = j < pd.N;
+      half_sync(h);  // the constants of the item before are read
+      if ((threadIdx.x & 127) < (unsigned)max(bk, 0)) {
+        const int e = threadIdx.x & 127;
+        const ModP m = a.mods[k0 + e];
+        ColConst &cq = cc[kHalf * h + e];
+        cq.p = m.p;
+        cq.pinv = m.pinv;
+        cq.r1 = m.r1;
+        cq.w48 = (uint32_t)(((uint64_t)m.r1 << 16) % m.p);
+      }
+      half_sync(h);
+      uint32_t res[kHalf];
+#pragma unroll
+      for (int e = 0; e < kHalf; ++e) res[e] = e < bk && live ? col[(size_t)e * S] : 0u;
+      // a failed wait: no more work, but the half's barriers go on
+      ok = __all_sync(0xffffffffu, ok && mbar_wait(b_accfull, n & 1, &abort_flag, a.err));
+      ++n;
+      if (!ok) continue;
+      tc_fence_after();
+#pragma unroll
+      for (int grp = 0; grp < 4; ++grp) {
+        uint32_t v[7][8];
+#pragma unroll
+        for (int k = 0; k < 7; ++k) tmem_ld8(tl + 32 * k + 8 * grp, v[k]);
+        asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+#pragma unroll
+        for (int k = 0; k < 7; ++k) tmem_hold8(v[k]);
+        if (grp == 3) {  // every class is in registers: free the accumulator
+#pragma unroll
+          for (int z = 0; z < 3; ++z) tmem_zero32(tl + 128 + 32 * z);
+          tmem_wait_st();
+          tc_fence_before();
+          __syncwarp();
+          if (lane == 0) mbar_arrive(b_accfree);
+        }
+#pragma unroll
+        for (int e = 0; e < 8; ++e) {
+          if (8 * grp + e >= bk) continue;
+          const ColConst &cq = cc[kHalf * h + 8 * grp + e];
+          const uint32_t val = window_value(v, e, cq);
+          if (live) col[(size_t)(8 * grp + e) * S] = msub(res[8 * grp + e], val, cq.p);
+        }
+      }
+    }
+  }
+  tc_fence_before();
+  __syncthreads();
+  if (warp == 8) {
+    tc_fence_after();
+    asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, 512;" ::"r"(tbase) : "memory");
+  }
+}
+
 // W digit tiles for blocks kb < KB: tile kb (kb - 1) / 2 + c (c < kb) holds
 // W[64 kb + 32 h + t][64 c + 32 u + e] (always l < k) as digit j, zero for
 // rows k >= K.  One thread per 16-byte row segment.
@@ -571,7 +754,15 @@ cudaError_t launch_g3m_rtiles(const int32_t *wtab, int K, int KB, uint16_t *out,
 }
 
 cudaError_t g3m_prepare() {
-  return cudaFuncSetAttribute(g3m_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmem);
+  cudaError_t e = cudaFuncSetAttribute(g3m_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmem);
+  if (e == cudaSuccess) e = cudaFuncSetAttribute(g3u_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 2 * kBuf);
+  return e;
+}
+
+cudaError_t launch_g3u(int sms, const G3uArgs &a, cudaStream_t s) {
+  const int items = a.ntasks * a.nkb;
+  if (items > 0) g3u_kernel<<<std::min(items, sms), kThreads, 2 * kBuf, s>>>(a);
+  return cudaGetLastError();
 }
 
 int64_t g3m_wtile_elems(int KB) { return KB > 1 ? (int64_t)KB * (KB - 1) / 2 * (2 * kBStage / 2) : 0; }

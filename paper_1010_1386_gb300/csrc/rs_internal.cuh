@@ -179,6 +179,21 @@ struct G3mArgs {
   const int32_t *stall;     // test hook: non-zero = the copy warp issues nothing
 };
 
+// Two-level CRT digits: the far products of one group of chunks (g3u_kernel).
+struct G3uArgs {
+  const PairDesc *pairs;
+  const int2 *tasks;        // (pair, first coefficient), coefficients in steps of 128
+  const ModP *mods;
+  const uint16_t *wtiles;   // W digit tiles per (block, chunk)
+  uint32_t *coef;           // residues, updated; digits below 64 c1
+  const uint16_t *xdig;     // operand digits of every task
+  const int64_t *xoff;      // per task: element offset of its operand digits
+  int32_t ntasks, c0, c1;   // chunks [c0, c1) of 64 digits go out of the blocks
+  int32_t nkb;              // kb in [c1, c1 + nkb)
+  int32_t *err;             // status word (a bounded wait ran out)
+  const int32_t *stall;     // test hook: non-zero = the copy warp issues nothing
+};
+
 // Tensor-core CRT limbs (kernels_g3l.cu): one block per (128 coefficients of
 // a pair, unit of 64 output limbs), over the 64-prime chunks whose prefix
 // products reach the unit; reads the digit rows the tensor-core digit kernel
@@ -257,6 +272,7 @@ struct G3Args {
   uint32_t *out;           // out: [coefficient][limb]
   int32_t *shape;          // out: per pair (1 + degree, limbs needed), zeroed before the launch
   int32_t kmax;            // largest K of the batch
+  int32_t kbeg = 0, kend = 0;  // tiled digits: of primes [kbeg, kend) only (kend 0: all), the products of digits below kbeg done
   int32_t signed_digits = 0;  // 1: the limbs come from the signed digits (no floor(P / 2) to remove)
 };
 
@@ -284,6 +300,7 @@ int64_t g3m_tile_elems(int K);
 cudaError_t launch_g3m_wtiles(const int32_t *wtab, int K, int KB, uint16_t *out, cudaStream_t s);
 int64_t g3m_rtile_elems(int KB);
 cudaError_t launch_g3m_rtiles(const int32_t *wtab, int K, int KB, uint16_t *out, cudaStream_t s);
+cudaError_t launch_g3u(int sms, const G3uArgs &a, cudaStream_t s);
 cudaError_t launch_g3m(int ntiles, const G3mArgs &a, cudaStream_t s);
 cudaError_t g3l_prepare();
 int64_t g3l_block_elems();  // bf16 elements of one (chunk, unit) block of prefix-product tiles
