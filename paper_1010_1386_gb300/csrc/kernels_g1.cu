@@ -312,6 +312,19 @@ __device__ __forceinline__ uint32_t reduce_coef(const uint32_t *src, int L, cons
   return acc;
 }
 
+// The same for many limbs (L <= 128): the products are summed exactly in 96
+// bits, one multiply a limb, and reduced once.
+__device__ __forceinline__ uint32_t reduce_long(const uint32_t *src, int L, const uint32_t *V, const ModP &m) {
+  uint32_t a0 = 0u, a1 = 0u, a2 = 0u;
+  for (int l = 0; l < L; ++l) rs_mac96(a0, a1, a2, src[l], V[l]);
+  uint64_t t = (uint64_t)a2 * m.r1 + a1;  // a2 < 2^7, 2^32 mod p <= 2^21: t < 2^32 + 2^28 < 3 p
+  if (t >= 2ull * m.p) t -= 2ull * m.p;
+  const uint32_t h = rs_umin((uint32_t)t, (uint32_t)t - m.p);
+  uint32_t acc = redc(((uint64_t)h << 32) | a0, m.p, m.pinv);
+  if (src[L - 1] >> 31) acc = msub(acc, redc((uint64_t)V[L], m.p, m.pinv), m.p);
+  return acc;
+}
+
 __device__ __forceinline__ int32_t signed_rep(uint32_t v, uint32_t p) {
   return v > (p >> 1) ? (int32_t)v - (int32_t)p : (int32_t)v;
 }
@@ -428,10 +441,55 @@ __device__ __forceinline__ void eval_chirp(uint32_t (&P)[C], const int32_t *sa, 
 }
 
 // Row k of the staged coefficients, k < 2 g1_half_rows(dx); qn[t] = q^{-C(t,2)}.
+// From 8 limbs the coefficients' products are summed before one reduction (for
+// 1 to 4 limbs that, or a choice inside the loop, costs 1 to 4% of the whole
+// kernel: hence a function of its own).  When long ones fill less than 40% of
+// the padded rows they are taken from a list of those that exist (column j's
+// start at smeta[j].x - smeta[0].x), so that a warp does not walk the limbs of
+// its few lanes that have one.  G1, us: 23,980 (pair, prime) items of 55 and 10
+// coefficients of 64 limbs 478 -> 343 (456 with the padded rows alone); 40,000
+// of 136 and 16 2,120 -> 1,868; 10,280 of those with 16 limbs 454 -> 442.
 template <int C>
-__device__ __forceinline__ void stage_chirp(int32_t *sa, const int2 *smeta, int deg, int dx,
+__device__ __noinline__ void stage_long(int32_t *sa, const int2 *smeta, int deg, int dx, int nc,
+                                        const uint32_t *limbs, int stride, int L,
+                                        const uint32_t *V, const uint32_t *qn, const ModP m) {
+  const int n = 2 * g1_half_rows(dx) * C, odd = g1_odd_offset(dx, C);
+  if (5 * nc >= 2 * n) {
+    for (int idx = threadIdx.x; idx < n; idx += blockDim.x) {
+      const int k = idx / C, r = idx - k * C, j = deg - r;
+      int32_t v = 0;
+      if (j >= 0 && k <= smeta[j].y)
+        v = signed_rep(mmul(reduce_long(limbs + ((size_t)k * stride + j) * L, L, V, m), qn[k], m), m.p);
+      sa[(k & 1) * odd + (k >> 1) * C + r] = v;
+    }
+    return;
+  }
+  for (int idx = threadIdx.x; idx < n; idx += blockDim.x) sa[(idx / C & 1) * odd + (idx / C >> 1) * C + idx % C] = 0;
+  __syncthreads();
+  for (int e = threadIdx.x; e < nc; e += blockDim.x) {
+    const int at = smeta[0].x + e;
+    int j = 0, hi = deg;  // the last column that starts at or before e: it has coefficients
+    while (j < hi) {
+      const int mid = (j + hi + 1) >> 1;
+      if (smeta[mid].x <= at)
+        j = mid;
+      else
+        hi = mid - 1;
+    }
+    const int k = at - smeta[j].x;
+    const uint32_t c = reduce_long(limbs + ((size_t)k * stride + j) * L, L, V, m);
+    sa[(k & 1) * odd + (k >> 1) * C + deg - j] = signed_rep(mmul(c, qn[k], m), m.p);
+  }
+}
+
+template <int C>
+__device__ __forceinline__ void stage_chirp(int32_t *sa, const int2 *smeta, int deg, int dx, int nc,
                                             const uint32_t *limbs, int stride, int L,
                                             const uint32_t *V, const uint32_t *qn, const ModP &m) {
+  if (L >= 8) {
+    stage_long<C>(sa, smeta, deg, dx, nc, limbs, stride, L, V, qn, m);
+    return;
+  }
   const int n = 2 * g1_half_rows(dx) * C, odd = g1_odd_offset(dx, C);
   for (int idx = threadIdx.x; idx < n; idx += blockDim.x) {
     const int k = idx / C, r = idx - k * C, j = deg - r;
@@ -475,8 +533,8 @@ __global__ void __launch_bounds__(128, RS_G1_MINB) g1_kernel(G1Args a) {
 
     for (int i = threadIdx.x; i < nmeta; i += blockDim.x) smeta[i] = a.meta[pd.meta_off + i];
     __syncthreads();
-    stage_chirp<C>(saf, smeta, pd.my, pd.mxf, a.limbs + pd.f_off, pd.fstride, pd.Lf, V, a.qn + tb, m);
-    stage_chirp<C>(sag, smeta + pd.my + 1, pd.ny, pd.mxg, a.limbs + pd.g_off, pd.gstride, pd.Lg, V,
+    stage_chirp<C>(saf, smeta, pd.my, pd.mxf, pd.fnc, a.limbs + pd.f_off, pd.fstride, pd.Lf, V, a.qn + tb, m);
+    stage_chirp<C>(sag, smeta + pd.my + 1, pd.ny, pd.mxg, pd.gnc, a.limbs + pd.g_off, pd.gstride, pd.Lg, V,
                    a.qn + tb, m);
     for (int i = threadIdx.x; i < 2 * (C / 8); i += blockDim.x) {
       const int w = i / (C / 8), top = (w ? pd.ny : pd.my) - 8 * (i - w * (C / 8));

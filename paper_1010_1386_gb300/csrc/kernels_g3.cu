@@ -379,15 +379,6 @@ __global__ void __launch_bounds__(128) g3p_kernel(G3Args a) {
 #endif
 constexpr int kG3bUnroll = RS_G3B_UNROLL;  // prime rows of the limb kernel per loop iteration
 
-// a2:a1:a0 += x * y (96-bit accumulator, one carry chain).
-__device__ __forceinline__ void mac96(uint32_t &a0, uint32_t &a1, uint32_t &a2, uint32_t x, uint32_t y) {
-  asm("mad.lo.cc.u32 %0, %3, %4, %0;\n\t"
-      "madc.hi.cc.u32 %1, %3, %4, %1;\n\t"
-      "addc.u32 %2, %2, 0;"
-      : "+r"(a0), "+r"(a1), "+r"(a2)
-      : "r"(x), "r"(y));
-}
-
 // Limb chunks: blockDim = 128 coefficients of one pair, one chunk of 16
 // output limbs.  With the offset digits w_k = v_k + (p_k - 1)/2 in [0, p_k)
 // the limb sums S[h] = sum_k w_k P_k[16 c + h] (P_k's 32-bit limbs) are
@@ -423,10 +414,10 @@ __global__ void __launch_bounds__(128) g3b_kernel(G3Args a) {
 #pragma unroll
     for (int q = 0; q < 4; ++q) {
       const uint4 l4 = __ldg(row + q);
-      mac96(a0[4 * q], a1[4 * q], a2[4 * q], w, l4.x);
-      mac96(a0[4 * q + 1], a1[4 * q + 1], a2[4 * q + 1], w, l4.y);
-      mac96(a0[4 * q + 2], a1[4 * q + 2], a2[4 * q + 2], w, l4.z);
-      mac96(a0[4 * q + 3], a1[4 * q + 3], a2[4 * q + 3], w, l4.w);
+      rs_mac96(a0[4 * q], a1[4 * q], a2[4 * q], w, l4.x);
+      rs_mac96(a0[4 * q + 1], a1[4 * q + 1], a2[4 * q + 1], w, l4.y);
+      rs_mac96(a0[4 * q + 2], a1[4 * q + 2], a2[4 * q + 2], w, l4.z);
+      rs_mac96(a0[4 * q + 3], a1[4 * q + 3], a2[4 * q + 3], w, l4.w);
     }
   }
   uint64_t carry = 0;

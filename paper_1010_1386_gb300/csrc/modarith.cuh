@@ -99,6 +99,15 @@ __device__ __forceinline__ int64_t rs_mac_s32(int64_t acc, int32_t a, int32_t b)
   return acc;
 }
 
+// a2:a1:a0 += x * y (96-bit accumulator, one carry chain).
+__device__ __forceinline__ void rs_mac96(uint32_t &a0, uint32_t &a1, uint32_t &a2, uint32_t x, uint32_t y) {
+  asm("mad.lo.cc.u32 %0, %3, %4, %0;\n\t"
+      "madc.hi.cc.u32 %1, %3, %4, %1;\n\t"
+      "addc.u32 %2, %2, 0;"
+      : "+r"(a0), "+r"(a1), "+r"(a2)
+      : "r"(x), "r"(y));
+}
+
 // hi 2^32 + lo -> hi c + lo for s = hi 2^32 + lo (c = 2^32 mod p, |c| < 2^31):
 // congruent mod p, and |result| < 2^31 |c| + 2^32.
 __device__ __forceinline__ int64_t rs_fold64(int64_t s, uint32_t c) {
