@@ -895,7 +895,13 @@ int rs_build_batch(rs_ctx *ctx, int n, const rs_bipoly *f, const rs_bipoly *g,
   // fewer than two per SM (few coefficients with many primes each).
   std::vector<int2> g3d;
   std::vector<int4> g3b;  // CRT limb chunks: 128 coefficients x one chunk per block
-  // Digits: one thread per coefficient when there are enough of them for one
+  // Everything in one kernel (g3f_kernel), one thread per coefficient, for at
+  // most 16 primes, and to 80 from 128 coefficients per SM; us before and so:
+  // 37 coefficients of 5 primes 13.6 and 9.9, 1,082 of 8 18.1 and 14.1, 129 of 18
+  // 20.1 and 20.0, 3,090 of 23 24.9 and 27.2, 10,178 of 42 36 and 48; 51,094 of 9
+  // 34.8 and 22.2, 24,994 of 32 52.9 and 36.8, 61,762 of 50 109 and 74, 245,084 of
+  // 72 541 and 516.
+  // Otherwise, digits: one thread per coefficient when there are enough of them for one
   // each to fill the GPU, the fewer the primes (a thread walks its K^2 / 2
   // products alone): from 96 per SM, 8 K per SM, 1024 per SM for any K.
   // Otherwise tiles of 32 or 16 coefficients on the CUDA cores, the tensor
@@ -945,6 +951,7 @@ int rs_build_batch(rs_ctx *ctx, int n, const rs_bipoly *f, const rs_bipoly *g,
       kc = std::max(kc, K);
       nk2 += (double)b->plans[i].N * K * K;
     }
+    b->g3_kc = kc;
     const int64_t sms = ctx->sms;
     b->g3_jt = nt32 < 2 * sms ? 16 : 32;
     b->g3_perthread = ncoef >= sms * std::min<int64_t>(RS_G3P_MIN_COEF_PER_SM, std::max(96, 8 * kc));
@@ -960,7 +967,9 @@ int rs_build_batch(rs_ctx *ctx, int n, const rs_bipoly *f, const rs_bipoly *g,
       ms_two += 0.004 + 0.009 * ((items + sms - 1) / sms);
       ++b->g3_nfar;
     }
-    const bool tc = !b->g3_perthread && !images_only && ctx->cfg.crt_form != 1;
+    b->g3_fused = !images_only && ctx->cfg.crt_form == 0 && kc > 0 &&
+                  (kc <= 16 || (kc <= RS_G3F_MAX_K && ncoef >= 128 * sms));
+    const bool tc = !b->g3_fused && !b->g3_perthread && !images_only && ctx->cfg.crt_form != 1;
     b->g3_two = tc && ctx->cfg.crt_form != 2 && b->g3_nfar > 0 && ms_two < ms_tiles &&
                 (kc < RS_G3M_MIN_K || ms_two < ms_tensor);
     if (!b->g3_two) b->g3_nfar = 0;
@@ -1011,7 +1020,8 @@ int rs_build_batch(rs_ctx *ctx, int n, const rs_bipoly *f, const rs_bipoly *g,
                             (b->nyun > 0) +
                             (b->ng3b > 0) +
                             (b->ng3 > 0);
-  b->info.kernel_launches += b->g3_two ? b->g3_nfar + ((maxK + 63) / 64 + 3) / 4 - 1 : 0;
+  if (b->g3_fused) b->info.kernel_launches -= (b->ng3d > 0) + (b->ng3b > 0);
+  b->info.kernel_launches += b->g3_two ? b->g3_nfar + (b->g3_kc + 255) / 256 - 1 : 0;
   for (const auto &gc : b->g2cls)
     if (gc.tensor) b->info.kernel_launches += 4;  // five launches per tensor-core class
 
@@ -1196,6 +1206,11 @@ int rs_build_batch(rs_ctx *ctx, int n, const rs_bipoly *f, const rs_bipoly *g,
       cudaError_t e2 = g2_prepare();
       if (e2 != cudaSuccess) rc = rs_fail(ctx, RS_ERR_CUDA, std::string("G2 set-up: ") + cudaGetErrorString(e2));
       ctx->g2_ready = e2 == cudaSuccess;
+    }
+    if (rc == RS_OK && b->g3_fused && !ctx->g3f_ready) {
+      cudaError_t e2 = g3f_prepare();
+      if (e2 != cudaSuccess) rc = rs_fail(ctx, RS_ERR_CUDA, std::string("CRT set-up: ") + cudaGetErrorString(e2));
+      ctx->g3f_ready = e2 == cudaSuccess;
     }
     for (auto &cl : b->classes) {
       if (rc != RS_OK) break;
@@ -1497,7 +1512,9 @@ static int enqueue(rs_batch *b, bool capturing) {
     a3.kmax = b->kmax;
     a3.signed_digits = b->g3_tlimbs ? 1 : 0;
     a3.xdig = b->g3_tlimbs ? b->d_g3m_x : nullptr;
-    if (b->g3_perthread) {
+    if (b->g3_fused) {
+      RS_CUDA(ctx, launch_g3f(b->ng3, b->g3_kc, a3, b->d_g3, s));
+    } else if (b->g3_perthread) {
       RS_CUDA(ctx, launch_g3p(b->ng3, a3, b->d_g3, s));
     } else if (b->g3_tensor) {
       G3mArgs am;
@@ -1533,7 +1550,7 @@ static int enqueue(rs_batch *b, bool capturing) {
       au.ntasks = b->ng3;
       au.err = reinterpret_cast<int32_t *>(b->d_out + b->status_off);
       au.stall = ctx->d_stall;
-      const int KB = (b->kmax + 63) / 64;
+      const int KB = (b->g3_kc + 63) / 64;
       for (int c = 0; c < KB; c += 4) {
         a3.kbeg = 64 * c;
         a3.kend = 64 * (c + 4);
@@ -1565,7 +1582,8 @@ static int enqueue(rs_batch *b, bool capturing) {
       RS_CUDA(ctx, launch_g3l(b->ng3b, al, s));
     }
     // the output kernel; the limb chunks unless the tensor cores formed the limbs
-    RS_CUDA(ctx, launch_g3bc(b->g3_tlimbs ? 0 : b->ng3b, b->ng3, b->g3_maxL, ctx->sms, a3, b->d_g3, s));
+    if (!b->g3_fused)
+      RS_CUDA(ctx, launch_g3bc(b->g3_tlimbs ? 0 : b->ng3b, b->ng3, b->g3_maxL, ctx->sms, a3, b->d_g3, s));
   }
   if (timing) RS_CUDA(ctx, record(b->ev[3], s, capturing));
   return RS_OK;

@@ -98,6 +98,7 @@ struct rs_ctx {
   int g3m_KB = 0;
   std::vector<void *> g3m_retired;
   bool g3m_ready = false;
+  bool g3f_ready = false;  // shared-memory attribute of the one-kernel Chinese remaindering set
   // Tensor-core CRT limbs: prefix-product tiles of the chunks c < g3l_KB,
   // block g3l_cbase[c] + u for the units u that chunk c reaches (host and
   // device copies of cbase; same lifetime rules, kept in g3m_retired).
@@ -170,9 +171,11 @@ struct rs_batch {
   int64_t status_off = 0; // word offset of the device status word (0 = every bounded wait completed)
   int ng2 = 0, ng3 = 0;
   int ng3d = 0, ng3b = 0, kmax = 0;  // CRT digit tiles, limb chunks, largest K
+  int g3_kc = 0;                     // largest prime count of the Chinese remaindering
   int g3_maxL = 0;                   // output limbs of the longest coefficients
   int g3_jt = 32;                    // coefficients per CRT digit tile (32 or 16)
   bool g3_perthread = false;         // CRT digits with one thread per coefficient
+  bool g3_fused = false;             // the whole Chinese remaindering in one kernel (few primes)
   bool g3_tensor = false;            // CRT digits on the tensor cores (kernels_g3m.cu)
   bool g3_two = false;               // CRT digits in two levels: tiles near, tensor cores far (g3u_kernel)
   int g3_nfar = 0;                   // launches of its far products

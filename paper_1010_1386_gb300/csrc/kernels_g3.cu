@@ -649,6 +649,153 @@ __global__ void __launch_bounds__(512) g3cp_kernel(G3Args a) {
   }
 }
 
+// The whole Chinese remaindering in one kernel for few primes (K <=
+// RS_G3F_MAX_K): a thread owns a coefficient as in g3p_kernel, keeps its digits
+// in a column of shared memory, forms each chunk of 16 limbs from them as in
+// g3b_kernel and removes floor(P / 2) and writes the chunk out as in
+// g3c_kernel, so neither digits nor limbs nor carries go through memory.
+// Shared memory: digits [K][128]; W by groups of four rows, W[4 g + i][l] at
+// 8 g (g - 1) + 4 l + i (l < 4 g: one 16-byte load gives four rows), then the
+// groups' 4 x 4 triangles.
+//
+// Bound by launch latency and the chain of digits for few coefficients, by the
+// products and the shared memory of a block for many.  Measured, against the
+// three kernels: see the choice of the digit kernels in engine.cu.
+__global__ void __launch_bounds__(128) g3f_kernel(G3Args a) {
+  extern __shared__ __align__(16) int32_t fsm[];
+  __shared__ ModP Ms[RS_G3F_MAX_K];
+  __shared__ uint32_t Cs[RS_G3F_MAX_K];
+  __shared__ uint32_t T[128 * 17];  // T[t * 17 + w]: limb 16 c + w of coefficient j0 + t
+  const int2 task = a.tasks[blockIdx.x];
+  const PairDesc pd = a.pairs[task.x];
+  const int K = pd.K, N = pd.N, S = pd.NI, t = (int)threadIdx.x, j0 = task.y, j = j0 + t;
+  const bool live = j < N;
+  const int L = pd.Lout, C = (L + 15) / 16, ng = (K + 3) >> 2;
+  int32_t *vs = fsm + t;                      // digit k at vs[128 k]
+  int32_t *Wq = fsm + 128 * K, *Wt = Wq + 8 * ng * (ng - 1);
+  const uint32_t *col = a.coef + pd.img_off + (live ? j : 0);
+#pragma unroll 4
+  for (int k = 0; k < K; ++k) vs[128 * k] = live ? (int32_t)col[(size_t)k * S] : 0;
+  for (int k = t; k < K; k += 128) {
+    Ms[k] = a.mods[k];
+    Cs[k] = a.crt[k];
+  }
+  for (int k = t >> 5; k < 4 * ng; k += 4) {
+    const int g = k >> 2, i = k & 3;
+    const int32_t *row = a.wtab + k * (k - 1) / 2;
+    for (int l = t & 31; l < 4 * g + 4; l += 32) {
+      const int32_t w = l < k && k < K ? __ldg(row + l) : 0;
+      if (l < 4 * g)
+        Wq[8 * g * (g - 1) + 4 * l + i] = w;
+      else
+        Wt[16 * g + 4 * i + l - 4 * g] = w;
+    }
+  }
+  __syncthreads();
+  for (int g = 0; g < ng; ++g) {  // digits, four rows at a time
+    const int k0 = 4 * g;
+    int64_t acc[4] = {0, 0, 0, 0};
+    const int4 *wq = reinterpret_cast<const int4 *>(Wq + 8 * g * (g - 1));
+    uint32_t c32[4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) c32[i] = Ms[min(k0 + i, K - 1)].r1;
+    int l = 0;
+    while (l < k0) {  // 4 products per fold: k0 is a multiple of 4
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        const int32_t v = vs[128 * (l + q)];
+        const int4 w = wq[l + q];
+        acc[0] = rs_mac_s32(acc[0], w.x, v);
+        acc[1] = rs_mac_s32(acc[1], w.y, v);
+        acc[2] = rs_mac_s32(acc[2], w.z, v);
+        acc[3] = rs_mac_s32(acc[3], w.w, v);
+      }
+      l += 4;
+#pragma unroll
+      for (int i = 0; i < 4; ++i) acc[i] = rs_fold64(acc[i], c32[i]);
+    }
+    int32_t vg[4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      if (k0 + i >= K) break;
+      const ModP m = Ms[k0 + i];
+      int64_t s2 = acc[i];  // |s2| < 2^53
+#pragma unroll
+      for (int c = 0; c < i; ++c) s2 = rs_mac_s32(s2, Wt[16 * g + 4 * i + c], vg[c]);  // + at most 3 products < 2^60
+      s2 = rs_fold64(s2, m.r1);
+      const uint32_t v = mmul(msub((uint32_t)vs[128 * (k0 + i)], finish64_3(s2, m), m.p), Cs[k0 + i], m);
+      vg[i] = signed_rep3(v, m.p);
+      vs[128 * (k0 + i)] = vg[i];
+    }
+  }
+  const int p0 = __ldg(a.poff + K);
+  const uint32_t *PK = reinterpret_cast<const uint32_t *>(a.p16 + p0);  // P's 32-bit limbs
+  const int plen = (__ldg(a.poff + K + 1) - p0) / 2;
+  uint32_t *o = a.out + pd.out_off;
+  int64_t r = 0;
+  int lo = 0, nz = 0, nf = 0;  // nz, nf: 2 (1 + last limb != 0, != 0xffffffff) + whether the sign needs one more
+  uint32_t top = 0u;
+  for (int c = 0; c < C; ++c) {
+    while (lo < K && __ldg(a.nh + lo) <= 32 * c) ++lo;  // prefix products below this chunk arrive as carries
+    uint32_t a0[16], a1[16], a2[16];
+#pragma unroll
+    for (int h = 0; h < 16; ++h) a0[h] = a1[h] = a2[h] = 0u;
+#pragma unroll 2
+    for (int k = lo; k < K; ++k) {
+      const uint32_t w = (uint32_t)(vs[128 * k] + (int32_t)((Ms[k].p - 1u) >> 1));
+      const uint4 *row = reinterpret_cast<const uint4 *>(a.p16 + __ldg(a.poff + k) + 32 * c);
+#pragma unroll
+      for (int q = 0; q < 4; ++q) {
+        const uint4 l4 = __ldg(row + q);
+        rs_mac96(a0[4 * q], a1[4 * q], a2[4 * q], w, l4.x);
+        rs_mac96(a0[4 * q + 1], a1[4 * q + 1], a2[4 * q + 1], w, l4.y);
+        rs_mac96(a0[4 * q + 2], a1[4 * q + 2], a2[4 * q + 2], w, l4.z);
+        rs_mac96(a0[4 * q + 3], a1[4 * q + 3], a2[4 * q + 3], w, l4.w);
+      }
+    }
+    uint64_t carry = 0;
+    uint32_t pk = 16 * c < plen ? __ldg(PK + 16 * c) : 0u;
+#pragma unroll
+    for (int w = 0; w < 16; ++w) {
+      const uint64_t lo64 = ((uint64_t)a1[w] << 32) | a0[w];
+      const uint64_t x = lo64 + carry;
+      carry = (x >> 32) + (((uint64_t)a2[w] + (x < lo64 ? 1u : 0u)) << 32);
+      const uint32_t pn = 16 * c + w + 1 < plen ? __ldg(PK + 16 * c + w + 1) : 0u;
+      const int64_t v = (int64_t)(uint32_t)x + r - (int64_t)((pk >> 1) | (pn << 31));
+      pk = pn;
+      const uint32_t limb = (uint32_t)v;
+      r = v >> 32;
+      T[t * 17 + w] = limb;
+      const int l = 16 * c + w;
+      if (l < L) {
+        if (limb != 0u) nz = 2 * (l + 1) + (int)(limb >> 31);
+        if (limb != 0xffffffffu) nf = 2 * (l + 1) + (int)(~limb >> 31);
+        top = limb;
+      }
+    }
+    r += (int64_t)carry;
+    __syncthreads();
+    const int nl = min(16, L - 16 * c);  // limbs of this chunk that exist
+#pragma unroll 4
+    for (int q = 0; q < 16; ++q) {
+      const int e = q * 128 + t, jj = e >> 4, w = e & 15;
+      if (j0 + jj < N && w < nl) o[(size_t)(j0 + jj) * L + 16 * c + w] = T[jj * 17 + w];
+    }
+    __syncthreads();
+  }
+  // fewest limbs whose two's-complement value is this coefficient
+  const bool neg = (top >> 31) != 0u;
+  const int code = neg ? nf : nz;
+  const bool zero = !live || (!neg && code == 0);
+  const int need = zero ? 0 : max(1, min((code >> 1) + (code & 1), L));
+  const int len = __reduce_max_sync(0xffffffffu, zero ? 0 : j + 1);
+  const int most = __reduce_max_sync(0xffffffffu, need);
+  if ((t & 31) == 0 && len) {
+    atomicMax(a.shape + 2 * task.x, len);
+    atomicMax(a.shape + 2 * task.x + 1, most);
+  }
+}
+
 // W[k][l] = p_0 ... p_{l-1} mod p_k (Montgomery form, signed), one thread per k.
 __global__ void crt_w_kernel(const ModP *mods, int K, int32_t *wtab) {
   const int k = blockIdx.x * blockDim.x + threadIdx.x;
@@ -729,6 +876,23 @@ cudaError_t launch_g3p(int nt, const G3Args &a, const int2 *tasks, cudaStream_t 
   G3Args at = a;
   at.tasks = tasks;
   if (nt) g3p_kernel<<<nt, 128, 0, s>>>(at);
+  return cudaGetLastError();
+}
+
+static size_t g3f_smem(int kmax) {
+  const int ng = (kmax + 3) / 4;
+  return (size_t)(128 * kmax + 8 * ng * (ng - 1) + 16 * ng) * 4;
+}
+
+cudaError_t g3f_prepare() {
+  return cudaFuncSetAttribute(g3f_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)g3f_smem(RS_G3F_MAX_K));
+}
+
+cudaError_t launch_g3f(int nc, int kmax, const G3Args &a, const int2 *otasks, cudaStream_t s) {
+  G3Args ao = a;
+  ao.tasks = otasks;
+  const size_t smem = g3f_smem(kmax);
+  if (nc) g3f_kernel<<<nc, 128, smem, s>>>(ao);
   return cudaGetLastError();
 }
 

@@ -10,6 +10,7 @@
 #define RS_G1_MAX_STAGED_WORDS (48 * 1024)  // staged residues + meta per G1 tile
 #define RS_G1_MAX_SMEM_BYTES (226 * 1024)  // of 227 KB, next to the kernel's static word
 #define RS_G2_PAD 8          // zero words around each G2 shared-memory region
+#define RS_G3F_MAX_K 80      // largest prime count of the one-kernel Chinese remaindering
 #define RS_CONV_R 7          // G2 outputs per register block; odd, so lanes hit distinct banks
 #define RS_G2_MAX_SMEM_BYTES (4 * (8192 + 2 * RS_G2_PAD) * 4)  // four regions of M <= 8192 pairs
 #define RS_NTT_LGMAX 13      // G2 transforms up to 2^13 points (N <= 2^12)
@@ -325,6 +326,8 @@ cudaError_t launch_yun(int ntasks, const YunArgs &a, cudaStream_t s);
 cudaError_t launch_g1s(int slots, int ntiles, size_t smem, const G1sArgs &a, cudaStream_t s);
 cudaError_t launch_g1s_fallback(int blocks, size_t smem, const G1sArgs &a, cudaStream_t s);
 cudaError_t launch_g2s(int ntasks, size_t smem, const G2sArgs &a, cudaStream_t s);
+cudaError_t g3f_prepare();
+cudaError_t launch_g3f(int nc, int kmax, const G3Args &a, const int2 *otasks, cudaStream_t s);
 cudaError_t launch_g3bc(int nb, int nc, int maxL, int sms, const G3Args &a, const int2 *otasks, cudaStream_t s);
 // Residues of one lifted factor divided by an integer g, prime by prime:
 // out[dst_off + k n + j] = in[src_off + k src_stride + j] * (g mod p_k)^{-1}
