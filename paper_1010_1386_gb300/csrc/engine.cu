@@ -1072,10 +1072,12 @@ int rs_build_batch(rs_ctx *ctx, int n, const rs_bipoly *f, const rs_bipoly *g,
   };
   const size_t o_in = carve(b->in_words * 4), o_meta = carve(meta.size() * sizeof(int2)),
                o_pairs = carve(b->descs.size() * sizeof(PairDesc)), o_tiles = carve(tiles.size() * sizeof(Tile)),
-               o_cnt = carve(16 * sizeof(int32_t)), o_num = carve(b->img_words * 4), o_den = carve(b->img_words * 4),
+               o_num = carve(b->img_words * 4), o_den = carve(b->img_words * 4),
                o_xl = carve(std::max(b->xl_words, b->out_words) * 4), o_out = carve(b->out_words * 4),
+               // after the results' shapes and status word: all that a pass zeroes, in one piece
+               o_cnt = carve(16 * sizeof(int32_t)), o_st = carve(ST_COUNT * sizeof(unsigned long long)),
                o_g2 = carve(g2.size() * sizeof(int2)), o_g3 = carve(g3.size() * sizeof(int2)),
-               o_st = carve(ST_COUNT * sizeof(unsigned long long)), o_cy = carve(b->cy_words * 8),
+               o_cy = carve(b->cy_words * 8),
                o_g3d = carve(g3d.size() * sizeof(int2)), o_yt = carve(yun.size() * sizeof(int2)),
                o_yo = carve((size_t)b->nyun * b->yun_ostride * 4), o_yw = carve((size_t)b->nyun * 8 * b->yun_wstride * 4),
                o_g3b = carve(g3b.size() * sizeof(int4)), o_fail = carve(b->schur ? b->img_words * sizeof(int2) : 0),
@@ -1303,10 +1305,10 @@ static int enqueue(rs_batch *b, bool capturing) {
     std::lock_guard<std::mutex> lock(ctx->tab_mu);
     tab = ctx->tab;
   }
-  RS_CUDA(ctx, cudaMemsetAsync(b->d_counters, 0, 16 * sizeof(int32_t), s));
-  RS_CUDA(ctx, cudaMemsetAsync(b->d_stats, 0, ST_COUNT * sizeof(unsigned long long), s));
-  if (b->g2t_x_elems > 0 || b->g3_tlimbs)  // the status word only the tensor-core kernels write
-    RS_CUDA(ctx, cudaMemsetAsync(b->d_out + b->status_off, 0, sizeof(uint32_t), s));
+  // Counters and statistics, and before them the results' shapes and status
+  // word: one launch (four of them were 4 us of a small call's 46).
+  char *const z0 = b->opt.images_only ? (char *)b->d_counters : (char *)(b->d_out + b->shape_off);
+  RS_CUDA(ctx, cudaMemsetAsync(z0, 0, (size_t)((char *)(b->d_stats + ST_COUNT) - z0), s));
   if (timing) RS_CUDA(ctx, record(b->ev[0], s, capturing));
   if (b->schur) {  // Schur variant of G1 over every tile, then the elimination fallback
     G1sArgs a;
@@ -1508,7 +1510,6 @@ static int enqueue(rs_batch *b, bool capturing) {
     a3.carry = b->d_cy;
     a3.out = b->d_out;
     a3.shape = reinterpret_cast<int32_t *>(b->d_out + b->shape_off);
-    RS_CUDA(ctx, cudaMemsetAsync(a3.shape, 0, b->descs.size() * 2 * sizeof(int32_t), s));
     a3.kmax = b->kmax;
     a3.signed_digits = b->g3_tlimbs ? 1 : 0;
     a3.xdig = b->g3_tlimbs ? b->d_g3m_x : nullptr;
