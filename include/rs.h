@@ -108,14 +108,14 @@ typedef struct {
   const char *autotune_cache;  /* tuner cache file merged at rs_create (a missing file is not an
                                   error) and rewritten at rs_destroy; NULL = none.  The string
                                   is copied. */
-  int32_t crt_form;          /* Chinese remaindering: 0 = by the batch's shape (digits with one
-                                thread per coefficient when there are at least 1024 coefficients
-                                per SM, fewer with few primes; else in tiles of coefficients on the
-                                CUDA cores or on the tensor cores, by an estimate of both; the
-                                limbs sum_k v_k P_k on the tensor cores when some pair has at least
-                                24 primes and the digits come in tiles), 1 = CUDA cores only,
-                                2 = digits and limbs on the tensor cores whenever the batch does
-                                not take one thread per coefficient */
+  int32_t crt_form;          /* Chinese remaindering: 0 = by the batch's shape (one kernel for few
+                                primes; else digits with one thread per coefficient when there are
+                                coefficients enough, in tiles of coefficients on the CUDA cores, on
+                                the tensor cores, or in both above 256 primes, by an estimate of
+                                each; the limbs sum_k v_k P_k on the tensor cores when some pair has
+                                at least 24 primes and the digits come in tiles), 1 = CUDA cores
+                                only, 2 = digits and limbs on the tensor cores whenever the batch
+                                does not take one thread per coefficient */
   int32_t reserved;          /* 0 */
 } rs_config;
 
