@@ -222,7 +222,8 @@ double rs_g2_cost(int N, int form) {
 // end.  Measured (us, G2 stage): 40,000 tasks of M = 113: 427 with 32 threads
 // (2 rounds, 3 segments), 474, 597, 986 and 1,599 with 64, 128, 256 and 512;
 // 546 of 2,049: 1,140, 1,027, 984 and 853 with 64, 128, 256 and 512; 69 of 451:
-// 20.2 with 384 threads in clusters, 24.2 with the best single blocks.
+// 20.2 with 384 threads in clusters, 24.2 with the best single blocks (all
+// before the first loads were taken together, which changed no order here).
 RsG2Shape rs_g2_shape(int M, int64_t tasks, int sms, const RsG2Shape *like) {
   static const int kT[8] = {32, 64, 96, 128, 192, 256, 384, 512};
   const int nblk = (M + RS_CONV_R - 1) / RS_CONV_R, npair = (nblk + 1) / 2, W = M + 2 * RS_G2_PAD;

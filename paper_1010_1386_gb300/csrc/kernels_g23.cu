@@ -147,9 +147,11 @@ __device__ __forceinline__ void pair_wait() { asm volatile("barrier.cluster.wait
 // steps around them), and for few tasks by a block's latency.  With one thread
 // per block pair and the halves in turn 3 to 33 lanes of a block worked;
 // splitting the walks fills them.  G2 stage, us, before (the fastest of the
-// three forms) -> now: 69 tasks of M = 451: 70 -> 20; 8,844 of 5 to 61: 83 ->
-// 37; 23,980 of 41: 248 -> 98; 10,280 of 113: 236 -> 119; 40,000 of 113: 860 ->
-// 427; 546 of 2,049: 880 -> 853; 1,127 of 169 to 1,369: 380 -> 268.
+// three forms) -> now: 69 tasks of M = 451: 70 -> 18; 8,844 of 5 to 61: 83 ->
+// 36; 23,980 of 41: 248 -> 96; 10,280 of 113: 236 -> 117; 40,000 of 113: 860 ->
+// 422; 546 of 2,049: 880 -> 853; 1,127 of 169 to 1,369: 380 -> 266.  Of these a
+// thread's first point's loads taken together at the start gave 20.4 -> 18.2
+// with 69 tasks and about 1% with 10,280 and more.
 __global__ void __launch_bounds__(512, 2) g2_kernel(G2Args a) {
   extern __shared__ __align__(16) uint32_t sm[];
   __shared__ uint32_t scratch[128];
@@ -169,24 +171,32 @@ __global__ void __launch_bounds__(512, 2) g2_kernel(G2Args a) {
   const uint32_t *finv = a.finv + tb, *gt = a.gtab + tb, *hq = a.hq + tb;
   const int32_t *bt = a.btab + tb;
 
+  // a thread's first point: its images and table entries, all on their way before the first is needed
+  const int f = min(tid, M - 1);
+  const uint32_t np0 = a.num[base + 2 * f], dp0 = a.den[base + 2 * f];
+  const uint32_t nm0 = a.num[base + 2 * f + 1], dm0 = a.den[base + 2 * f + 1];
+  const uint32_t fi0 = finv[f], hq0 = hq[f], hqe = hq[0], gt0 = gt[f];
+  const int32_t bt0 = bt[f];
   uint32_t *dens = reinterpret_cast<uint32_t *>(Bs);
-  for (int i = tid; i < M; i += T) dens[i] = mmul(a.den[base + 2 * i], a.den[base + 2 * i + 1], m);
+  if (tid < M) dens[tid] = mmul(dp0, dm0, m);
+  for (int i = tid + T; i < M; i += T) dens[i] = mmul(a.den[base + 2 * i], a.den[base + 2 * i + 1], m);
   __syncthreads();
   batch_invert(dens, Y, M, m, scratch, true);  // plain inverses: from here on plain times Montgomery form
   __syncthreads();
   for (int i = tid; i < M; i += T) {
-    const uint32_t np = a.num[base + 2 * i], dp = a.den[base + 2 * i];
-    const uint32_t nm = a.num[base + 2 * i + 1], dm = a.den[base + 2 * i + 1];
-    const uint32_t fy = mmul(finv[i], Y[i], m);
+    const bool f0 = i < T;
+    const uint32_t np = f0 ? np0 : a.num[base + 2 * i], dp = f0 ? dp0 : a.den[base + 2 * i];
+    const uint32_t nm = f0 ? nm0 : a.num[base + 2 * i + 1], dm = f0 ? dm0 : a.den[base + 2 * i + 1];
+    const uint32_t fy = mmul(f0 ? fi0 : finv[i], Y[i], m);
     for (int h = 0; h < nh; ++h) {
       const bool odd = (h0 + h) != 0;
       const uint32_t v = mmul2(np, dm, odd ? mneg(nm, m.p) : nm, dp, m);  // z+ +- z-
       // E / F_i or O / F_i; hq[0] = 1/2
-      X[h * W + i] = signed_rep(mmul(mmul(v, hq[odd ? i : 0], m), fy, m), m.p);
+      X[h * W + i] = signed_rep(mmul(mmul(v, odd ? (f0 ? hq0 : hq[i]) : hqe, m), fy, m), m.p);
     }
   }
   if (split) pair_arrive();
-  for (int i = tid; i < M; i += T) Bs[i] = bt[i];
+  for (int i = tid; i < M; i += T) Bs[i] = i < T ? bt0 : bt[i];
   for (int i = tid; i < RS_G2_PAD; i += T) {
     for (int h = 0; h < nh; ++h) {
       X[h * W - 1 - i] = 0;
@@ -201,18 +211,22 @@ __global__ void __launch_bounds__(512, 2) g2_kernel(G2Args a) {
     int32_t *x = X + hh * W;
     conv_parts(x, Bs, Y, cs, hc, W, m);  // Y: Q^{C(k,2)} c_k
     __syncthreads();
-    for (int k = tid; k < M; k += T)
+    for (int k = tid; k < M; k += T) {
+      const uint32_t g = k < T ? gt0 : gt[k];
       for (int h = 0; h < hc; ++h)
-        x[h * W + D - k] = signed_rep(mmul(conv_value(Y, cs, h, k, m), gt[k], m), m.p);  // c_k F_k reversed
+        x[h * W + D - k] = signed_rep(mmul(conv_value(Y, cs, h, k, m), g, m), m.p);  // c_k F_k reversed
+    }
     __syncthreads();
     conv_parts(x, Bs, Y, cs, hc, W, m);  // Y[D - t]: sum_s c_{t+s} F_{t+s} b_s
     __syncthreads();
     if (split) pair_wait();
-    for (int i = tid; i < M; i += T)
+    for (int i = tid; i < M; i += T) {
+      const uint32_t fi = i < T ? fi0 : finv[i];
       for (int h = 0; h < hc; ++h) {
         const int c = 2 * i + h0 + hh + h;
-        if (c < N) a.coef[base + c] = mmul(conv_value(Y, cs, h, D - i, m), finv[i], m);
+        if (c < N) a.coef[base + c] = mmul(conv_value(Y, cs, h, D - i, m), fi, m);
       }
+    }
     __syncthreads();
   }
 }
