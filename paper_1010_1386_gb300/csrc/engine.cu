@@ -690,11 +690,8 @@ int rs_build_batch(rs_ctx *ctx, int n, const rs_bipoly *f, const rs_bipoly *g,
   std::vector<int2> g2, g3;
   std::vector<int> byN(order);
   std::sort(byN.begin(), byN.end(), [&](int x, int y) { return b->plans[x].N > b->plans[y].N; });
-  // G2 launches by point count: each thread owns one pair of output blocks
-  // of the convolutions per round; a (pair, prime) gets the fewest rounds
-  // with at most 256 threads, and the fewest warps for them, so the threads
-  // of a block carry equal work (classes of 32, 64, ..., 256 threads).
-  // Pairs whose transform-based G2 is cheaper go to one launch per transform
+  // G2 launches: the direct form by octaves of point counts, shaped by
+  // rs_g2_shape.  Pairs whose transform-based G2 is cheaper go to one launch per transform
   // length instead (256 threads, shared memory 3 N + 2^lg words).
   // The form is chosen per transform-length group: forced by the context or
   // the options, else the tuner's cached choice (timed now when missing and

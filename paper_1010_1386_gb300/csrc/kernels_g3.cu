@@ -16,7 +16,9 @@
 //      in 96-bit carry chains and normalises the chunk, keeping its carry.
 // G3c: one block per 128 coefficients ripples the chunk carries, subtracts
 //      floor(P/2) = sum_k (p_k - 1)/2 P_k and writes the two's-complement
-//      32-bit limbs through shared memory in coalesced runs.
+//      32-bit limbs through shared memory in coalesced runs; G3cp: the same
+//      with the chunks of few, long coefficients in parallel.
+// G3f: all of it in one kernel for few primes.
 #include <algorithm>
 
 #include "../../include/rs.h"
