@@ -465,13 +465,13 @@ void rs_free_batch(rs_batch *b) {
   delete b;
 }
 
-void rs_batch_sizes(const std::vector<PairPlan> &plans, const rs_bipoly *f, const rs_bipoly *g,
-                    int64_t *in_words, int64_t *out_words, int64_t *device_bytes) {
+void rs_batch_sizes(const std::vector<PairPlan> &plans, int64_t *in_words, int64_t *out_words,
+                    int64_t *device_bytes) {
   int64_t in = 0, out = 0, img = 0, meta = 0, tiles = 0, g2 = 0, g3 = 0, xl = 0, cy = 0, g3d = 0, g3b = 0;
   int64_t t_items = 0, t_bytes = 0;  // tensor-core G2 work items and buffers, if every pair takes that form
   for (size_t i = 0; i < plans.size(); ++i) {
-    in += rs_input_words(f[i]) + rs_input_words(g[i]);
     const PairPlan &p = plans[i];
+    in += rs_used_words(p, p.f) + rs_used_words(p, p.g);
     if (p.status != RS_OK || p.trivial_zero) continue;
     const int64_t chunks = (p.Lout + 15) / 16;
     out += (int64_t)p.N * p.Lout + 2;
@@ -521,11 +521,11 @@ int rs_build_batch(rs_ctx *ctx, int n, const rs_bipoly *f, const rs_bipoly *g,
   b->in_g.assign(n, -1);
   int maxM = 1, maxK = 0, maxDx = 0;  // largest point-pair count, prime count, x-degree
   for (int i = 0; i < n; ++i) {
-    b->in_f[i] = b->in_words;
-    b->in_words += rs_input_words(f[i]);
-    b->in_g[i] = b->in_words;
-    b->in_words += rs_input_words(g[i]);
     const PairPlan &p = b->plans[i];
+    b->in_f[i] = b->in_words;
+    b->in_words += rs_used_words(p, p.f);
+    b->in_g[i] = b->in_words;
+    b->in_words += rs_used_words(p, p.g);
     if (p.status != RS_OK || p.trivial_zero) continue;
     PairDesc d;
     memset(&d, 0, sizeof(d));
@@ -1258,8 +1258,10 @@ int rs_upload(rs_batch *b, const rs_bipoly *f, const rs_bipoly *g) {
   const int step = std::max(1, b->n / 64);
   ctx->pool.run((b->n + step - 1) / step, threads, [&](int t) {
     for (int i = t * step; i < std::min(b->n, (t + 1) * step); ++i) {
-      memcpy(b->h_in + b->in_f[i], f[i].coeffs, rs_input_words(f[i]) * 4);
-      memcpy(b->h_in + b->in_g[i], g[i].coeffs, rs_input_words(g[i]) * 4);
+      const PairPlan &p = b->plans[i];
+      if (p.status != RS_OK || p.trivial_zero) continue;
+      memcpy(b->h_in + b->in_f[i], f[i].coeffs, rs_used_words(p, p.f) * 4);
+      memcpy(b->h_in + b->in_g[i], g[i].coeffs, rs_used_words(p, p.g) * 4);
     }
   });
   if (b->in_words)

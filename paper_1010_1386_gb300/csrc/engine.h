@@ -245,8 +245,8 @@ RsG2Shape rs_g2_shape(int M, int64_t tasks, int sms, const RsG2Shape *like);
 int rs_build_batch(rs_ctx *ctx, int n, const rs_bipoly *f, const rs_bipoly *g,
                    std::vector<PairPlan> &&plans, const RsBatchOpts &opt, rs_batch **out);
 // Byte sizes a batch of these plans needs (device arena, host staging in/out).
-void rs_batch_sizes(const std::vector<PairPlan> &plans, const rs_bipoly *f, const rs_bipoly *g,
-                    int64_t *in_words, int64_t *out_words, int64_t *device_bytes);
+void rs_batch_sizes(const std::vector<PairPlan> &plans, int64_t *in_words, int64_t *out_words,
+                    int64_t *device_bytes);
 int rs_upload(rs_batch *b, const rs_bipoly *f, const rs_bipoly *g);
 int rs_run(rs_batch *b);
 int rs_fetch_async(rs_batch *b);                                // enqueue the result copy

@@ -40,6 +40,15 @@ struct PairPlan {
 int rs_plan_pair(const rs_bipoly *f, const rs_bipoly *g, const std::vector<double> &log2p,
                  PairPlan &plan, const char **why);
 
+// Words of p's coefficient array that a batch uploads: the rows up to its true
+// x-degree (an array padded with zero rows has the plan of the trimmed one, so
+// a reused batch may meet either).  None for a pair that was rejected, whose
+// array is not looked at again, or whose resultant is trivially zero.
+inline int64_t rs_used_words(const PairPlan &plan, const PolyInfo &p) {
+  if (plan.status != RS_OK || plan.trivial_zero) return 0;
+  return (int64_t)(p.mx + 1) * p.stride * p.L;
+}
+
 // Words of per-j x-degrees, chirp-scaled coefficients of f and g ([x-degree +
 // 1][C] each) and the window of q^{C(t,2)} for a tile of `threads` points: the
 // measure the planner's limit on staged inputs is stated in.

@@ -187,7 +187,7 @@ void launch(RsServer *s, std::unique_lock<std::mutex> &lk) {
     plans[i] = take[i]->plan;
   }
   int64_t in_w = 0, out_w = 0, dev_b = 0;
-  rs_batch_sizes(plans, F.data(), G.data(), &in_w, &out_w, &dev_b);
+  rs_batch_sizes(plans, &in_w, &out_w, &dev_b);
   int rc = grow_pinned(s->h_in[slot], s->h_in_words[slot], in_w);
   if (rc == RS_OK) rc = grow_pinned(s->h_out[slot], s->h_out_words[slot], out_w);
   RsBatchOpts o;
@@ -382,7 +382,7 @@ int rs_server_submit(rs_ctx *ctx, const rs_bipoly *f, const rs_bipoly *g, uint64
   r->g.coeffs = r->gl.data();
   int64_t in_w, out_w, dev_b;
   std::vector<PairPlan> one(1, r->plan);
-  rs_batch_sizes(one, &r->f, &r->g, &in_w, &out_w, &dev_b);
+  rs_batch_sizes(one, &in_w, &out_w, &dev_b);
   r->footprint = dev_b;
   {
     std::lock_guard<std::mutex> lk(s->mu);
