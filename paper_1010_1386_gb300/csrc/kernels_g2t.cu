@@ -74,6 +74,7 @@ __global__ void __launch_bounds__(kThreads, 1) g2t_gemm_kernel(G2tArgs a) {
   __shared__ __align__(8) uint64_t bar[10];  // full[2], empty[2], accfull[2], accfree[2], drain
   __shared__ uint32_t tmem_slot;
   __shared__ volatile int abort_flag;
+  __shared__ int late;  // a wait ran out before this block
   const G2tItem it = a.items[blockIdx.x];
   const G2tRowTile rt = a.rts[it.rt];
   const ModP m = a.mods[rt.prime];
@@ -84,6 +85,7 @@ __global__ void __launch_bounds__(kThreads, 1) g2t_gemm_kernel(G2tArgs a) {
   const uint32_t b_accfull = smem_u32(&bar[4]), b_accfree = smem_u32(&bar[6]), b_drain = smem_u32(&bar[8]);
   if (threadIdx.x == 0) {
     abort_flag = 0;
+    late = gave_up(a.err);
     for (int i = 0; i < 2; ++i) {
       mbar_init(b_full + 8 * i, 1);
       mbar_init(b_empty + 8 * i, 1);
@@ -102,6 +104,11 @@ __global__ void __launch_bounds__(kThreads, 1) g2t_gemm_kernel(G2tArgs a) {
   __syncthreads();
   tc_fence_after();
   const uint32_t tbase = tmem_slot;
+  if (late) {
+    if (warp == 8)
+      asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, 512;" ::"r"(tbase) : "memory");
+    return;
+  }
 
   // Register split (launch: 168 per thread, 64,512 in all): the control
   // warpgroup gives back down to 88, the two draining warpgroups take 208

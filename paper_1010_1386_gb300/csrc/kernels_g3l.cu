@@ -85,6 +85,7 @@ __global__ void __launch_bounds__(kThreads, 1) g3l_kernel(G3lArgs a) {
   __shared__ __align__(8) uint64_t bar[13];  // full[4], empty[4], accfull[2], accfree[2], done
   __shared__ uint32_t tmem_slot;
   __shared__ volatile int abort_flag;
+  __shared__ int late;  // a wait ran out before this block
   __shared__ int32_t qs[128];  // buffer 1's carries out of column 255, per row
   const int4 lt = a.ltasks[blockIdx.x];
   const int2 task = a.tasks[lt.x];
@@ -99,6 +100,7 @@ __global__ void __launch_bounds__(kThreads, 1) g3l_kernel(G3lArgs a) {
   const uint32_t b_accfull = smem_u32(&bar[8]), b_accfree = smem_u32(&bar[10]), b_done = smem_u32(&bar[12]);
   if (threadIdx.x == 0) {
     abort_flag = 0;
+    late = gave_up(a.err);
     for (int i = 0; i < kStages; ++i) {
       mbar_init(b_full + 8 * i, 1);
       mbar_init(b_empty + 8 * i, 1);
@@ -119,6 +121,11 @@ __global__ void __launch_bounds__(kThreads, 1) g3l_kernel(G3lArgs a) {
   __syncthreads();
   tc_fence_after();
   const uint32_t tbase = tmem_slot;
+  if (late) {
+    if (warp == 8)
+      asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, 512;" ::"r"(tbase) : "memory");
+    return;
+  }
 
   // Sub-stages in order: chunk lo + ci, stage s = 2 (32-prime half) + digit
   // pair; g counts them and picks the buffer (g % 4) and the phases.

@@ -133,6 +133,7 @@ __global__ void __launch_bounds__(kThreads, 1) g3m_kernel(G3mArgs a) {
   __shared__ __align__(8) uint64_t bar[12];
   __shared__ uint32_t tmem_slot;
   __shared__ volatile int abort_flag;
+  __shared__ int late;  // a wait ran out before this block
   // Constants of the block's primes: half 0's 32 (used by half 0 only) and
   // half 1's 32 by block parity (half 0 fills them for the next block while
   // half 1 still uses this block's).
@@ -153,6 +154,7 @@ __global__ void __launch_bounds__(kThreads, 1) g3m_kernel(G3mArgs a) {
   const uint32_t b_a1 = smem_u32(&bar[11]);
   if (threadIdx.x == 0) {
     abort_flag = 0;
+    late = gave_up(a.err);
     for (int i = 0; i < 2; ++i) {
       mbar_init(b_full + 8 * i, 1);
       mbar_init(b_empty + 8 * i, 1);
@@ -174,6 +176,11 @@ __global__ void __launch_bounds__(kThreads, 1) g3m_kernel(G3mArgs a) {
   __syncthreads();
   tc_fence_after();
   const uint32_t tbase = tmem_slot;
+  if (late) {
+    if (warp == 8)
+      asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, 512;" ::"r"(tbase) : "memory");
+    return;
+  }
 
   // Register split (launch: 168 per thread, 64,512 in all): the control
   // warpgroup gives back down to 72, the draining warpgroups take 216 each
@@ -529,6 +536,7 @@ __global__ void __launch_bounds__(kThreads, 1) g3u_kernel(G3uArgs a) {
   __shared__ __align__(8) uint64_t bar[7];  // full[2], empty[2], accfull, accfree, drain
   __shared__ uint32_t tmem_slot;
   __shared__ volatile int abort_flag;
+  __shared__ int late;  // a wait ran out before this block
   __shared__ ColConst cc[kBlkK];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const uint32_t sbase = smem_u32(sm);
@@ -536,6 +544,7 @@ __global__ void __launch_bounds__(kThreads, 1) g3u_kernel(G3uArgs a) {
   const uint32_t b_accfull = smem_u32(&bar[4]), b_accfree = smem_u32(&bar[5]), b_drain = smem_u32(&bar[6]);
   if (threadIdx.x == 0) {
     abort_flag = 0;
+    late = gave_up(a.err);
     for (int i = 0; i < 2; ++i) {
       mbar_init(b_full + 8 * i, 1);
       mbar_init(b_empty + 8 * i, 1);
@@ -554,6 +563,11 @@ __global__ void __launch_bounds__(kThreads, 1) g3u_kernel(G3uArgs a) {
   __syncthreads();
   tc_fence_after();
   const uint32_t tbase = tmem_slot;
+  if (late) {
+    if (warp == 8)
+      asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, 512;" ::"r"(tbase) : "memory");
+    return;
+  }
   const int items = a.ntasks * a.nkb;
   // pair and digit block of an item; false when the pair has no such block
   auto item_of = [&](int it, int &t, int &kb) {

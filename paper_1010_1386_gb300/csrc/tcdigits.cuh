@@ -71,6 +71,12 @@ __device__ bool mbar_wait(uint32_t bar, uint32_t parity, volatile int *abort, in
   }
 }
 
+// Whether a wait has run out before this block started, in an earlier launch of
+// the pass or an earlier block of this one: the block then returns at its first
+// barrier, so that the waits of a pass run out once, not once per launch and
+// wave.  For thread 0 before that barrier: the answer has to be the block's.
+__device__ __forceinline__ int gave_up(const int32_t *err) { return *(const volatile int32_t *)err; }
+
 __device__ __forceinline__ void bulk_load(uint32_t dst, const void *src, uint32_t bytes, uint32_t bar) {
   asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(dst),
                "l"(src), "r"(bytes), "r"(bar)

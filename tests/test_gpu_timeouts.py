@@ -48,3 +48,26 @@ def test_crt_digit_wait_runs_out_and_context_recovers():
     assert rs.result_bound(*pairs[0])["primes"] > 64  # two digit blocks: the copy warp has work
     with rs.Context(device=0, crt_form=2) as c:
         _expect_timeout_then_recover(c, pairs)
+
+
+@pytest.mark.parametrize("what,form,n,dx,dy,bits", [
+    ("two-level digits: four far launches, then the limbs", dict(crt_form=0), 1, 1, 5, 3700),
+    ("digits in more blocks than the GPU holds, then the limbs", dict(crt_form=2), 200, 1, 2, 700),
+    ("interpolation in more blocks than the GPU holds, twice", dict(g2_form=4), 2, 20, 4, 800),
+])
+def test_one_wait_a_pass(what, form, n, dx, dy, bits):
+    """Launches and blocks after the first wait that ran out (a second) do not
+    take a second each."""
+    rng = random.Random(63)
+    pairs = [tuple(rs.as_bipoly(rand_bipoly(rng, dx, dy, bits)) for _ in range(2)) for _ in range(n)]
+    with rs.Context(device=0, **form) as c:
+        want = c.resultant_batch(pairs)
+        c.stall_tensor_cores(True)
+        t0 = time.time()
+        with pytest.raises(rs.RsError) as ei:
+            c.resultant_batch(pairs)
+        took = time.time() - t0
+        c.stall_tensor_cores(False)
+        assert ei.value.code == RS_ERR_TIMEOUT
+        assert 0.9 < took < 1.9
+        assert c.resultant_batch(pairs) == want
