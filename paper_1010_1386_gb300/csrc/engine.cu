@@ -18,6 +18,25 @@ thread_local std::string g_err;
 constexpr size_t kAlign = 256;
 size_t align_up(size_t x) { return (x + kAlign - 1) & ~(kAlign - 1); }
 
+// Whether G1 evaluates plan p (register capacity C) through its threads'
+// columns of shared memory: unless they leave an SM room for one block of 128
+// threads (or none, at C = 72) where the staged coefficients alone leave room
+// for two.  G1, ns per image, degrees in x and y of f and g; before there were
+// columns, with them, without:
+//   (300, 71) (1, 8)    1 and 2 blocks    3.61   4.36   3.14
+//   (400, 55) (1, 12)   1 and 2           3.10   3.88   2.63
+//   (660, 71) (1, 4)    none and 1        8.99   14.5 (64 threads)   8.03
+//   (200, 38) (200, 38) 2 and 3           2.15   1.97   1.94
+//   (250, 30) (250, 30) 2 and 3           1.99   1.81   1.71
+//   (150, 44) (150, 44) 2 and 3           2.24   2.12   2.19
+//   (150, 38) (150, 38) 3 and 4           1.81   1.49   1.54
+//   (100, 70) (100, 70) 2 and 2           3.76   3.03   3.32
+//   (500, 71) (1, 8)    1 and 1           6.85   5.70   6.09
+static bool rs_g1_column(const PairPlan &p, int C) {
+  auto blocks = [&](bool col) { return (227 * 1024) / (rs_g1_smem_words(p, C, 128, col) * 4 + 1024); };
+  return blocks(true) > 1 || blocks(true) == blocks(false);
+}
+
 // Modular products of the normal remainder sequence (a4 count): three per
 // coefficient of a double step, two of the single step between equal degrees.
 double prs_products(int a, int b) {
@@ -603,12 +622,14 @@ int rs_build_batch(rs_ctx *ctx, int n, const rs_bipoly *f, const rs_bipoly *g,
   // else the tuner's cached choice (timed now when missing and allowed), else
   // 128 points on a persistent grid.
   std::vector<Tile> tiles;
-  for (int cap = 8; cap <= 72; cap += 8) {
+  for (int v = 0; v < 18; ++v) {  // capacities 8 .. 72, with the column and without
+    const int cap = 8 * (v / 2 + 1);
+    const bool col = v % 2 == 0;
     std::vector<int> members;
     int cmaxN = 0;
     int64_t cimages = 0;
     for (int i : order)
-      if (g1_supported_cap(b->plans[i].cap) == cap) {
+      if (g1_supported_cap(b->plans[i].cap) == cap && rs_g1_column(b->plans[i], cap) == col) {
         members.push_back(i);
         cmaxN = std::max(cmaxN, b->plans[i].N);
         cimages += (int64_t)b->plans[i].K * b->plans[i].N;
@@ -631,13 +652,10 @@ int rs_build_batch(rs_ctx *ctx, int n, const rs_bipoly *f, const rs_bipoly *g,
     }
     ch.persistent = (ch.persistent && opt.persistent) ? 1 : 0;
     if (opt.g1_threads > 0 || ctx->cfg.tile_points > 0) ch.persistent = opt.persistent ? 1 : 0;
-    // The per-thread columns and the staged coefficients of the largest accepted
-    // inputs exceed a block's shared memory with 128 threads at C = 72.
-    int T = ch.threads;
-    for (int i : members)
-      while (T > 32 && rs_g1_smem_words(b->plans[i], cap, T) * 4 > RS_G1_MAX_SMEM_BYTES) T >>= 1;
+    const int T = ch.threads;
     RsClassLaunch cl;
     cl.cap = cap;
+    cl.col = col;
     cl.threads = T;
     cl.persistent = ch.persistent;
     cl.tile_off = (int64_t)tiles.size();
@@ -651,7 +669,7 @@ int rs_build_batch(rs_ctx *ctx, int n, const rs_bipoly *f, const rs_bipoly *g,
     for (int i : members) {
       const PairPlan &p = b->plans[i];
       cl.cost += (double)p.K * p.N * (p.f.nc + p.g.nc + 2.0 * p.f.my * p.g.my);
-      cl.smem = std::max(cl.smem, (size_t)rs_g1_smem_words(p, cap, T) * 4);
+      cl.smem = std::max(cl.smem, (size_t)rs_g1_smem_words(p, cap, T, col) * 4);
       const int M = (p.N + 1) / 2;  // point pairs: two threads each
       for (int k = 0; k < p.K; ++k) {
         if (ctx->cfg.univariate == 0) {
@@ -1073,7 +1091,7 @@ int rs_build_batch(rs_ctx *ctx, int n, const rs_bipoly *f, const rs_bipoly *g,
                o_num = carve(b->img_words * 4), o_den = carve(b->img_words * 4),
                o_xl = carve(std::max(b->xl_words, b->out_words) * 4), o_out = carve(b->out_words * 4),
                // after the results' shapes and status word: all that a pass zeroes, in one piece
-               o_cnt = carve(16 * sizeof(int32_t)), o_st = carve(ST_COUNT * sizeof(unsigned long long)),
+               o_cnt = carve(RS_G1_COUNTERS * sizeof(int32_t)), o_st = carve(ST_COUNT * sizeof(unsigned long long)),
                o_g2 = carve(g2.size() * sizeof(int2)), o_g3 = carve(g3.size() * sizeof(int2)),
                o_cy = carve(b->cy_words * 8),
                o_g3d = carve(g3d.size() * sizeof(int2)), o_yt = carve(yun.size() * sizeof(int2)),
@@ -1214,13 +1232,13 @@ int rs_build_batch(rs_ctx *ctx, int n, const rs_bipoly *f, const rs_bipoly *g,
     }
     for (auto &cl : b->classes) {
       if (rc != RS_OK) break;
-      const int64_t key = ((int64_t)cl.cap << 40) | ((int64_t)cl.threads << 24) | (int64_t)((cl.smem + 1023) / 1024);
+      const int64_t key = ((int64_t)cl.cap << 40) | ((int64_t)cl.col << 39) | ((int64_t)cl.threads << 24) | (int64_t)((cl.smem + 1023) / 1024);
       auto it = ctx->g1_occupancy.find(key);
       int mb = 0;
       if (it != ctx->g1_occupancy.end()) {
         mb = it->second;
       } else {
-        cudaError_t e2 = g1_prepare(cl.cap, cl.threads, ((cl.smem + 1023) / 1024) * 1024, &mb);
+        cudaError_t e2 = g1_prepare(cl.cap, cl.col, cl.threads, ((cl.smem + 1023) / 1024) * 1024, &mb);
         if (e2 != cudaSuccess) {
           rc = rs_fail(ctx, RS_ERR_CUDA, std::string("G1 set-up: ") + cudaGetErrorString(e2));
           break;
@@ -1322,7 +1340,7 @@ static int enqueue(rs_batch *b, bool capturing) {
     a.num = b->d_num;
     a.den = b->d_den;
     a.fail = b->d_fail;
-    a.fail_count = b->d_counters + 15;
+    a.fail_count = b->d_counters + RS_G1_COUNTERS - 1;
     a.stats = b->d_stats;
     RS_CUDA(ctx, launch_g1s(b->schur_slots, b->ntiles_all, b->schur_smem, a, s));
     RS_CUDA(ctx, launch_g1s_fallback(2 * ctx->sms, b->schur_fb_smem, a, s));
@@ -1350,7 +1368,7 @@ static int enqueue(rs_batch *b, bool capturing) {
     cudaError_t fe = cudaSuccess;
     cudaStream_t si = branch_begin(b, 0, ci - 1, s, &fe);
     RS_CUDA(ctx, fe);
-    RS_CUDA(ctx, launch_g1(cl.cap, cl.threads, cl.blocks, cl.smem, a, si));
+    RS_CUDA(ctx, launch_g1(cl.cap, cl.col, cl.threads, cl.blocks, cl.smem, a, si));
     branch_end(b, 0, ci - 1, si, &fe);
     RS_CUDA(ctx, fe);
   }

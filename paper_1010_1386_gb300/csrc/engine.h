@@ -109,8 +109,11 @@ struct rs_ctx {
   bool g3l_ready = false;
 };
 
+#define RS_G1_COUNTERS 32
+
 struct RsClassLaunch {
   int cap = 0;
+  bool col = true;  // values through a shared column per thread, or not (inputs with many coefficients)
   int threads = 128;
   int persistent = 1;
   double cost = 0.0;  // modular products of the class (launch order: costliest first)
@@ -203,7 +206,7 @@ struct rs_batch {
   int2 *d_meta = nullptr;
   PairDesc *d_pairs = nullptr;
   Tile *d_tiles = nullptr;
-  int32_t *d_counters = nullptr;
+  int32_t *d_counters = nullptr;  // RS_G1_COUNTERS: a tile counter per G1 launch, the last the Schur variant's failures
   uint32_t *d_num = nullptr, *d_den = nullptr, *d_xl = nullptr, *d_out = nullptr;
   int2 *d_g2 = nullptr, *d_g3 = nullptr;
   unsigned long long *d_stats = nullptr;

@@ -359,6 +359,12 @@ __device__ __forceinline__ int32_t signed_rep(uint32_t v, uint32_t p) {
 //   rolled   0.265  0.363  0.512  0.742  0.978  1.237  1.593  1.845
 // Signed sums that start at 0 (8 rows before the first fold) measured 1-3%
 // slower beyond 8 rows and 2% faster up to them.
+//
+// The columns are (C + 1) words a thread.  Inputs whose staged coefficients
+// leave too little room beside them (the rule and both sides' times: engine.cu,
+// rs_g1_column) take the form without (COL false): the same loop, each block's
+// values selected into the register array; at most two blocks fit an SM then,
+// so a thread may have 255 registers.
 
 // Rows of one parity of a polynomial of x-degree mx (both parities have the
 // same number; the last row may be a zero row), and the distance in words
@@ -376,8 +382,8 @@ __host__ __device__ __forceinline__ int g1_poly_words(int mx, int C) { return g1
 // The sign of the second is the same for every coefficient of f and g; the
 // image takes it back.  sa: staged coefficients of this lane's parity; steps:
 // rows per block of 8 columns; win: the window at this point pair and parity;
-// col: this thread's C words of shared memory.
-template <int C>
+// col: this thread's C words of shared memory (COL).
+template <int C, bool COL>
 __device__ __forceinline__ void eval_chirp(uint32_t (&P)[C], const int32_t *sa, const int32_t *steps,
                                            const int32_t *win, uint32_t *col, int par, const ModP &m) {
   const uint32_t c32 = m.r1;  // 2^32 mod p
@@ -432,12 +438,21 @@ __device__ __forceinline__ void eval_chirp(uint32_t (&P)[C], const int32_t *sa, 
       const uint32_t h = (uint32_t)(acc[r] >> 32);  // < 15 2^28 + 2^21 < 2 p
       const uint32_t v = redc(((uint64_t)rs_umin(h, h - m.p) << 32) | (uint32_t)acc[r], m.p, m.pinv);
       const uint32_t s = v + __shfl_xor_sync(0xffffffffu, v * sg + off, 1);  // < 2 p
-      pc[r] = rs_umin(s, s - m.p);
+      const uint32_t z = rs_umin(s, s - m.p);
+      if constexpr (COL) {
+        pc[r] = z;
+      } else {
+#pragma unroll
+        for (int q = 0; q < C; q += 8)
+          if (q == 8 * b) P[q + r] = z;
+      }
     }
     pc += 8;
   }
+  if constexpr (COL) {
 #pragma unroll
-  for (int r = 0; r < C; ++r) P[r] = col[r];
+    for (int r = 0; r < C; ++r) P[r] = col[r];
+  }
 }
 
 // Row k of the staged coefficients, k < 2 g1_half_rows(dx); qn[t] = q^{-C(t,2)}.
@@ -500,8 +515,8 @@ __device__ __forceinline__ void stage_chirp(int32_t *sa, const int2 *smeta, int 
   }
 }
 
-template <int C>
-__global__ void __launch_bounds__(128, RS_G1_MINB) g1_kernel(G1Args a) {
+template <int C, bool COL>
+__global__ void __launch_bounds__(128, COL ? RS_G1_MINB : 2) g1_kernel(G1Args a) {
   extern __shared__ __align__(16) uint32_t sm[];
   __shared__ int s_tile;
   bool first = true;
@@ -528,7 +543,7 @@ __global__ void __launch_bounds__(128, RS_G1_MINB) g1_kernel(G1Args a) {
     int32_t *saf = reinterpret_cast<int32_t *>(sm) + ((2 * nmeta + 2 * (C / 8) + 7) & ~7);  // 32-byte aligned
     int32_t *sag = saf + ((g1_poly_words(pd.mxf, C) + 7) & ~7);
     int32_t *swin = sag + g1_poly_words(pd.mxg, C);
-    uint32_t *scol = reinterpret_cast<uint32_t *>(swin) + (blockDim.x >> 1) + dxm + 2 + threadIdx.x * (C + 1);  // odd stride
+    uint32_t *scol = reinterpret_cast<uint32_t *>(swin) + (blockDim.x >> 1) + dxm + 2 + threadIdx.x * (C + 1);  // odd stride; with COL
     const size_t tb = (size_t)tl.prime * a.tstride;
 
     for (int i = threadIdx.x; i < nmeta; i += blockDim.x) smeta[i] = a.meta[pd.meta_off + i];
@@ -565,8 +580,8 @@ __global__ void __launch_bounds__(128, RS_G1_MINB) g1_kernel(G1Args a) {
       // every thread evaluates (the shuffles need the whole warp); only the
       // threads of the chunk's pairs run the remainder sequence
       uint32_t A[C], B[C];
-      eval_chirp<C>(A, saf + par * g1_odd_offset(pd.mxf, C), ssteps, swin + ti + par, scol, par, m);
-      eval_chirp<C>(B, sag + par * g1_odd_offset(pd.mxg, C), ssteps + C / 8, swin + ti + par, scol, par, m);
+      eval_chirp<C, COL>(A, saf + par * g1_odd_offset(pd.mxf, C), ssteps, swin + ti + par, scol, par, m);
+      eval_chirp<C, COL>(B, sag + par * g1_odd_offset(pd.mxg, C), ssteps + C / 8, swin + ti + par, scol, par, m);
       if (ti < nn) {
         unlucky = (A[0] == 0u || B[0] == 0u) ? 1u : 0u;
         Prs s;
@@ -607,21 +622,21 @@ __global__ void __launch_bounds__(128, RS_G1_MINB) g1_kernel(G1Args a) {
 #define RS_CAT2(a, b) a##b
 #define RS_CAT(a, b) RS_CAT2(a, b)
 
-cudaError_t RS_CAT(rs_g1_launch_, RS_G1_CAP)(int threads, int blocks, size_t smem, const G1Args &a,
+cudaError_t RS_CAT(rs_g1_launch_, RS_G1_CAP)(bool col, int threads, int blocks, size_t smem, const G1Args &a,
                                             cudaStream_t s) {
-  g1_kernel<RS_G1_CAP><<<blocks, threads, smem, s>>>(a);
+  if (col)
+    g1_kernel<RS_G1_CAP, true><<<blocks, threads, smem, s>>>(a);
+  else
+    g1_kernel<RS_G1_CAP, false><<<blocks, threads, smem, s>>>(a);
   return cudaGetLastError();
 }
 
-cudaError_t RS_CAT(rs_g1_prepare_, RS_G1_CAP)(int threads, size_t smem, int *mb) {
-  const size_t smem_used = smem;
+cudaError_t RS_CAT(rs_g1_prepare_, RS_G1_CAP)(bool col, int threads, size_t smem, int *mb) {
   // The attribute is per kernel, not per launch: always allow the largest
   // staging any plan may request so that batches prepared earlier with more
   // shared memory keep working.
-  (void)smem;
-  cudaError_t e = cudaFuncSetAttribute(g1_kernel<RS_G1_CAP>,
-                                       cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       RS_G1_MAX_SMEM_BYTES);
+  const void *k = col ? (const void *)g1_kernel<RS_G1_CAP, true> : (const void *)g1_kernel<RS_G1_CAP, false>;
+  cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, RS_G1_MAX_SMEM_BYTES);
   if (e != cudaSuccess) return e;
-  return cudaOccupancyMaxActiveBlocksPerMultiprocessor(mb, g1_kernel<RS_G1_CAP>, threads, smem_used);
+  return cudaOccupancyMaxActiveBlocksPerMultiprocessor(mb, k, threads, smem);
 }

@@ -61,9 +61,9 @@ inline int rs_g1_staged_words(const PairPlan &p, int C, int threads) {
 // Shared-memory words of a G1 tile of `threads` points of plan p in
 // register-capacity class C, an upper bound: the above with the rows split by
 // parity (a row and up to 31 words more per polynomial), the row counts per
-// block of 8 columns, and one column of C + 1 words per thread.
-inline int rs_g1_smem_words(const PairPlan &p, int C, int threads) {
-  return rs_g1_staged_words(p, C, threads) + 2 * (C + 31 + 8) + 2 * (C / 8) + 8 + (C + 1) * threads;
+// block of 8 columns, and with `col` one column of C + 1 words per thread.
+inline int rs_g1_smem_words(const PairPlan &p, int C, int threads, bool col) {
+  return rs_g1_staged_words(p, C, threads) + 2 * (C + 31 + 8) + 2 * (C / 8) + 8 + (col ? (C + 1) * threads : 0);
 }
 
 // Primes in (2^31 - 2^20, 2^31), descending, by a sieve of Eratosthenes.

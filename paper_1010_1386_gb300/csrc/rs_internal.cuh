@@ -278,9 +278,9 @@ struct G3Args {
 };
 
 // Launchers (kernels_*.cu).  Each returns the cudaGetLastError() of its launch.
-cudaError_t launch_g1(int cap, int threads, int blocks, size_t smem, const G1Args &a, cudaStream_t s);
+cudaError_t launch_g1(int cap, bool col, int threads, int blocks, size_t smem, const G1Args &a, cudaStream_t s);
 int g1_supported_cap(int cap);           // smallest compiled register capacity >= cap, or 0
-cudaError_t g1_prepare(int cap, int threads, size_t smem, int *max_blocks_per_sm);
+cudaError_t g1_prepare(int cap, bool col, int threads, size_t smem, int *max_blocks_per_sm);
 cudaError_t launch_g2(int threads, int blocks, size_t smem, const G2Args &a, cudaStream_t s);
 cudaError_t g2_prepare();
 cudaError_t g2n_prepare();

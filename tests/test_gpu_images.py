@@ -4,13 +4,13 @@ matrix, over degrees at the edges of the register capacities and phases,
 equal, adjacent and far apart, on dense inputs and on sparse ones whose
 sequence meets vanishing pivots; the evaluation's row groups (7 products per
 fold, two parities) at their edges, with zero coefficients and inputs so large
-that a block takes fewer threads."""
+that the evaluation takes no shared columns."""
 import random
 
 import pytest
 
 from oracle import modp
-from tests.helpers import rand_bipoly
+from tests.helpers import check_sampled_31, rand_bipoly
 
 pytestmark = pytest.mark.gpu
 
@@ -92,3 +92,22 @@ def test_largest_staged_inputs(ctx):
     little shared memory for 128 threads' columns."""
     rng = random.Random(9)
     check(ctx, rand_bipoly(rng, 470, 71, 12), rand_bipoly(rng, 190, 1, 12), primes=1, points=4)
+
+
+@pytest.mark.parametrize("cap", range(8, 80, 8))
+def test_without_columns(ctx, cap):
+    """About 28,100 words staged: two blocks of 128 threads fit an SM's shared
+    memory without their columns (28,800 words each), one with them."""
+    rng = random.Random(cap)
+    dx = 27900 // (cap + 1) - 8
+    check(ctx, rand_bipoly(rng, dx, cap - 1, 12), rand_bipoly(rng, 3, 1, 12), primes=1, points=70)
+
+
+def test_both_forms_of_a_capacity():
+    """One batch with pairs of the same register capacity in both forms."""
+    from paper_1010_1386_gb300 import rs
+    rng = random.Random(12)
+    pairs = [(rand_bipoly(rng, dx, 39, 12), rand_bipoly(rng, 2, 2, 12)) for dx in (3, 672, 5, 672, 17)]
+    with rs.Context() as c:
+        for (f, g), R in zip(pairs, c.resultant_batch(pairs)):
+            check_sampled_31(f, g, R, rng)
