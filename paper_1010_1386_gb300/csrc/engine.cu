@@ -926,16 +926,25 @@ int rs_build_batch(rs_ctx *ctx, int n, const rs_bipoly *f, const rs_bipoly *g,
   // cores of all SMs; whichever these times (ms, fitted to the measurements
   // below; 608 schedulers' products against one tile's chain of digit blocks
   // per wave, and for two levels both a group's chain and its waves of far
-  // products) say.  Limbs: on the tensor cores unless the digits took one
-  // thread per coefficient or no pair has 24 primes.
+  // products) say, each with its limbs' time.  Limbs: on the CUDA cores after
+  // one thread per coefficient; on the tensor cores after digits there; after
+  // tiles on the CUDA cores too, unless a pair has 24 primes and these times
+  // say otherwise: a thread's chain over the longest pair's primes or the
+  // products of all, against 8 us a block (128 coefficients of a pair and 64
+  // limbs, mostly the read-out, however few the coefficients) and 1 us a
+  // 64-prime chunk, one block per SM.  With tensor-core limbs from 24 primes on,
+  // one long pair took thousands of short ones there.  CRT stage, us, CUDA-core
+  // and tensor-core limbs: 4,183 pairs of 97 coefficients and 6 primes with 4 of
+  // 1,117 and 116 264 and 467; 1,216 of 55 and 6 with one of 949 and 69 84 and 175;
+  // 4,305 of 13 and 52 with 8 of 13 and 790 807 and 891; 359 of 13 and 6 with one
+  // of 9 and 63 44 and 51; 288 of 9 and 16 with one of 33 and 219 100 and 59; 822
+  // of 9 and 7 with 2 of 9 and 735 675 and 539 (in 70 mixed batches the estimates'
+  // choice was at most 6% slower than the other).
   // CRT stage, us: CUDA-core tiles with CUDA-core limbs, with tensor-core
   // limbs, tensor-core digits and limbs, one thread per coefficient (with the
   // digits' earlier kernel, which took one warp through each digit block's 64
   // steps, the first column was 79, 727, 694, 1,650 and 5,910 us in rows 3, 6,
   // 8, 10 and 11):
-  // Two levels, against the fastest of the others with the carry kernel of
-  // kernels_g3.cu: 4,097 of 546 229 -> 184, 4,520 of 514 232 -> 190, 1,640 of
-  // 1,199 504 -> 307, 4,520 of 2,000 2,028 -> 1,003, 63,008 of 526 1,792 -> 1,772.
   //   coefficients  primes (avg)  tiles  + limbs  tensor  per thread
   //     1,160         27             24      22      43      41
   //     3,178          8             24      24      43      30
@@ -955,12 +964,18 @@ int rs_build_batch(rs_ctx *ctx, int n, const rs_bipoly *f, const rs_bipoly *g,
   //    50,782         22             59      76              47
   //    24,994         32             49      53              55
   //   116,878         32            134     170              92
+  // Two levels, against the fastest of the others with the carry kernel of
+  // kernels_g3.cu: 4,097 of 546 229 -> 184, 4,520 of 514 232 -> 190, 1,640 of
+  // 1,199 504 -> 307, 4,520 of 2,000 2,028 -> 1,003, 63,008 of 526 1,792 -> 1,772.
   {
     int64_t nt32 = 0, nt128 = 0, ncoef = 0;
     int kc = 0;  // largest prime count of the Chinese remaindering
-    double nk2 = 0.0;
+    double nk2 = 0.0, limb_work = 0.0, limb_tc = 0.0;  // limbs: products on the CUDA cores; us of blocks on the tensor cores
     for (int i : order) {
-      const int K = b->descs[b->dev_index[i]].K;
+      const int K = b->descs[b->dev_index[i]].K, L = b->plans[i].Lout, kb = (K + 63) / 64, units = (L + 63) / 64;
+      limb_work += 0.25 * ((b->plans[i].N + 31) / 32) * ((L + 15) / 16) * K;
+      // unit u takes about kb - u of the pair's kb chunks: 64 primes are 62 limbs
+      limb_tc += (double)((b->plans[i].N + 127) / 128) * (8.0 * units + 0.5 * std::min(kb, units) * (2 * kb + 1 - std::min(kb, units)));
       nt32 += (b->plans[i].N + 31) / 32;
       nt128 += (b->plans[i].N + 127) / 128;
       ncoef += b->plans[i].N;
@@ -986,12 +1001,15 @@ int rs_build_batch(rs_ctx *ctx, int n, const rs_bipoly *f, const rs_bipoly *g,
     b->g3_fused = !images_only && ctx->cfg.crt_form == 0 && kc > 0 &&
                   (kc <= 16 || (kc <= RS_G3F_MAX_K && ncoef >= 128 * sms));
     const bool tc = !b->g3_fused && !b->g3_perthread && !images_only && ctx->cfg.crt_form != 1;
-    b->g3_two = tc && ctx->cfg.crt_form != 2 && b->g3_nfar > 0 && ms_two < ms_tiles &&
+    const double ms_climbs = std::max(2.1e-4 * kc, 2.3e-7 * limb_work * 152 / sms), ms_tlimbs = 1e-3 * limb_tc / sms;
+    const bool tlimbs = kc >= RS_G3L_MIN_K && ms_tlimbs < ms_climbs;  // after tiles
+    const double ms_cuda = ms_tiles + (tlimbs ? ms_tlimbs : ms_climbs);
+    b->g3_two = tc && ctx->cfg.crt_form != 2 && b->g3_nfar > 0 && ms_two + ms_tlimbs < ms_cuda &&
                 (kc < RS_G3M_MIN_K || ms_two < ms_tensor);
     if (!b->g3_two) b->g3_nfar = 0;
-    b->g3_tensor =
-        tc && !b->g3_two && (ctx->cfg.crt_form == 2 || (kc >= RS_G3M_MIN_K && ms_tensor < ms_tiles));
-    b->g3_tlimbs = tc && (b->g3_tensor || b->g3_two || kc >= RS_G3L_MIN_K);
+    b->g3_tensor = tc && !b->g3_two &&
+                   (ctx->cfg.crt_form == 2 || (kc >= RS_G3M_MIN_K && ms_tensor + ms_tlimbs < ms_cuda));
+    b->g3_tlimbs = tc && (b->g3_tensor || b->g3_two || tlimbs);
   }
   for (int i : order) {
     const PairPlan &p = b->plans[i];

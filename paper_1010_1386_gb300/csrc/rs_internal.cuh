@@ -161,7 +161,7 @@ struct G2tArgs {
 #define RS_G2T_MAX_M 4096  // point pairs per (pair, prime) the tensor-core form takes
 
 #define RS_G3M_MIN_K 128  // largest prime count from which a batch's digits may take the tensor cores
-#define RS_G3L_MIN_K 24   // ... and from which its limbs do
+#define RS_G3L_MIN_K 24   // ... and from which its limbs may
 
 // Tensor-core CRT digits (kernels_g3m.cu): one block per 128 coefficients of
 // one pair (the output kernel's tasks), over 64-prime digit blocks.

@@ -80,3 +80,18 @@ def test_one_thread_per_coefficient_with_few_primes():
         got = ctx.resultant_batch(pairs)
     for i in range(0, 900, 29):
         assert got[i] == exact.resultant_y(*pairs[i])
+
+
+@pytest.mark.parametrize("n,bits", [(40, 900), (1500, 900), (1500, 2300)])  # limbs on the tensor cores, then on the CUDA cores twice
+def test_one_long_pair(n, bits):
+    """One pair of about 120 or 300 primes with many of a few."""
+    from paper_1010_1386_gb300 import rs
+    rng = random.Random(n + bits)
+    pairs = [(rand_bipoly(rng, 2, 2, 20), rand_bipoly(rng, 2, 2, 20)) for _ in range(n)]
+    pairs.insert(n // 2, (rand_bipoly(rng, 6, 2, bits), rand_bipoly(rng, 6, 2, bits)))
+    with rs.Context() as ctx:
+        got = ctx.resultant_batch(pairs)
+    for i in [n // 2] + list(range(0, n, 97)):
+        assert got[i] == exact.resultant_y(*pairs[i])
+    with rs.Context(crt_form=1) as ctx:
+        assert ctx.resultant_batch(pairs) == got
