@@ -2124,7 +2124,7 @@ int rs_resultant_y(rs_ctx *ctx, const rs_bipoly *f, const rs_bipoly *g, rs_upoly
 // would reject is passed through unchanged so that it fails the same way.
 static rs_bipoly transposed(const rs_bipoly &p, std::vector<uint32_t> &buf) {
   if (!p.coeffs || p.deg_x < 0 || p.deg_y < 0 || p.limbs < 1 || p.limbs > RS_MAX_LIMBS ||
-      (int64_t)(p.deg_x + 1) * (p.deg_y + 1) > ((int64_t)1 << 26))
+      ((int64_t)p.deg_x + 1) * ((int64_t)p.deg_y + 1) > ((int64_t)1 << 26))
     return p;
   const int nx = p.deg_x + 1, ny = p.deg_y + 1, L = p.limbs;
   buf.resize((size_t)nx * ny * L);

@@ -154,7 +154,7 @@ int analyze(const rs_bipoly *f, PolyInfo &pi, const char **why) {
     *why = "limbs must be in 1..RS_MAX_LIMBS (128)";
     return RS_ERR_ARG;
   }
-  if ((int64_t)(f->deg_x + 1) * (f->deg_y + 1) > ((int64_t)1 << 26)) {
+  if (((int64_t)f->deg_x + 1) * ((int64_t)f->deg_y + 1) > ((int64_t)1 << 26)) {
     *why = "input array too large";
     return RS_ERR_LIMIT;
   }

@@ -211,6 +211,20 @@ def test_create_without_gpu_fails_cleanly(lib):
     assert e.value.code == -4
 
 
+@pytest.mark.parametrize("field", ["deg_x", "deg_y"])
+@pytest.mark.parametrize("value", [2**31 - 1, 2**31 - 2, 2**26])
+def test_largest_extents_are_refused(lib, field, value):
+    """deg + 1 is taken in 64 bits (no coefficient of such an array is read)."""
+    f = rs._Polys([[[1, 2], [3, 4]]])
+    g = rs._Polys([[[1, 2], [3, 4]]])
+    for P in (f, g):
+        keep = int(P.raw[0][field])
+        P.raw[0][field] = value
+        assert lib.rs_result_bound(f.structs, g.structs, None, None, None, None) == -6
+        P.raw[0][field] = keep
+    assert lib.rs_result_bound(f.structs, g.structs, None, None, None, None) == 0
+
+
 def test_autotune_cache_file_roundtrip(lib, tmp_path):
     """The tuner cache is host state: a file merges into it, is written back
     in the same form, and a malformed line rejects the whole file."""
