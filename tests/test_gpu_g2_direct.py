@@ -48,3 +48,15 @@ def test_largest_counts(direct, dx, dy):
     rng = random.Random(dx)
     f, g = rand_bipoly(rng, dx, dy, 6), rand_bipoly(rng, dx, dy, 6)
     check_sampled_31(f, g, direct.resultant_y(f, g), rng)
+
+
+@pytest.mark.parametrize("dx", [820, 812])
+def test_largest_counts_with_many_primes(direct, dx):
+    """More than two blocks per SM: the halves in turn (6,561 point pairs), and
+    both at once at the shared-memory limit (6,497)."""
+    from paper_1010_1386_gb300 import rs
+    rng = random.Random(dx)
+    f, g = rand_bipoly(rng, dx, 8, 650), rand_bipoly(rng, dx, 8, 650)
+    assert rs.result_bound(f, g)["primes"] > 304
+    R = direct.resultant_y(f, g)
+    check_sampled_31(f, g, R, rng)
