@@ -39,3 +39,33 @@ def test_carries(form, chunks, n):
             want = exact.resultant_y(f, g)
             assert max(abs(x) for x in want) >> s == 2**top - 1
             assert ctx.resultant_y(f, g) == want
+
+
+@pytest.mark.parametrize("bits", [984, 1000, 1496, 1900, 2200, 2430])
+def test_carries_in_one_kernel(bits):
+    """The same values in the one-kernel remaindering, 2 to 5 chunks of 16 limbs
+    (up to 80 primes), which many coefficients take."""
+    from paper_1010_1386_gb300 import rs
+    rng = random.Random(bits)
+    special = [0, 1, -1]
+    for b in range(8, bits, 8):
+        special += [2**b, 2**b - 1, 1 - 2**b, -(2**b), -(2**b) - 1, 2**b + 1]
+    pairs, want = [], []
+    for i in range(100):
+        cs = [(1 - 2 * (i & 1)) * (2**bits - 1)] + [rng.choice(special) for _ in range(298)] + [1]
+        f, g, _ = scaled_pair(cs, 0)
+        pairs.append((f, g))
+        want.append(cs)
+    sign = exact.resultant_y(*pairs[0])[299]
+    want = [[sign * c for c in cs] for cs in want]
+    assert want[1] == exact.resultant_y(*pairs[1])
+    launches = []
+    for form in (0, 1):
+        with rs.Context(crt_form=form) as ctx:
+            b = ctx.batch(pairs)
+            b.run()
+            b.sync()
+            assert b.results() == want
+            launches.append(b.info()["kernel_launches"])
+            b.close()
+    assert launches[0] == launches[1] - 2
