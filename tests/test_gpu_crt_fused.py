@@ -48,12 +48,18 @@ def test_few_primes(K):
 
 @pytest.mark.parametrize("K", [17, 18, 32, 33, 34, 63, 66, 79, 80])
 def test_more_primes(K):
+    from paper_1010_1386_gb300 import rs
     rng = random.Random(K)
     _, _, bits = pair_with_primes(rng, 12, K)
-    pairs = [(rand_bipoly(rng, 12, 1, bits), rand_bipoly(rng, 12, 1, bits)) for _ in range(1000)]  # 25,000 coefficients
+    pairs = []
+    while len(pairs) < 1000:  # 25,000 coefficients
+        f, g = rand_bipoly(rng, 12, 1, bits), rand_bipoly(rng, 12, 1, bits)
+        if rs.result_bound(f, g)["primes"] <= K:  # some ask for one prime more than the probe's
+            pairs.append((f, g))
+    assert max(rs.result_bound(f, g)["primes"] for f, g in pairs) == K
     got, launches = run(pairs)
     tiles, more = run(pairs, form=1)
     assert got == tiles
-    assert launches < more or K > 78  # the bound of a few pairs may ask for one prime more than the probe's
+    assert launches < more
     for i in range(0, len(pairs), 97):
         assert got[i] == exact.resultant_y(*pairs[i])
