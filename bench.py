@@ -299,18 +299,29 @@ def int_peak():
     return _PEAK
 
 
-def roofline(info, g1_ms, clk, kernel="G1 (reduce + evaluate + univariate resultant)"):
-    """G1's algorithmic IMAD rate (4 multiply-adds per modular product of
-    the evaluation and the remainder sequence) against the measured
-    mad.lo.u32 peak of this device."""
+# 32-bit integer multiply-adds that G1 executes per modular product (a wide one
+# counts as two, a Montgomery reduction is a low and a wide one), evaluation and
+# resultant.  Remainder sequence: lazy sums, one wide product each (the folds and
+# the reduction per coefficient, below a tenth, are left out), and double steps,
+# three products and one reduction.  Schur variant: Horner steps, and two products
+# per reduction.
+G1_MADS = {"prs": (2.0, 3.0), "schur": (5.0, 3.5)}
+
+
+def roofline(info, g1_ms, clk, kernel="G1 (reduce + evaluate + univariate resultant)", univariate="prs"):
+    """G1's rate of executed multiply-adds (G1_MADS per modular product of the
+    evaluation and the resultants) against the measured mad.lo.u32 peak of this
+    device; beside it the rate at the conventional four per product."""
     pk = int_peak()
     peak = pk["mad_lo_u32"] / 1e12
-    achieved = 4.0 * (info["modmul_eval"] + info["modmul_prs"]) / (g1_ms * 1e-3) / 1e12
+    ev, res = G1_MADS[univariate]
+    achieved = (ev * info["modmul_eval"] + res * info["modmul_prs"]) / (g1_ms * 1e-3) / 1e12
+    four = 4.0 * (info["modmul_eval"] + info["modmul_prs"]) / (g1_ms * 1e-3) / 1e12
     sm_max = clk["sm_max_mhz"] or pk["clock_max_mhz"]
     derived = pk["sms"] * IMAD_PER_SM_CLK * sm_max * 1e6 / 1e12
     return {"bound": "alu", "kernel": kernel,
             "achieved": achieved, "peak": peak, "unit": "TIMAD/s", "frac": achieved / peak,
-            "traffic": None,
+            "at_four_per_product": four, "traffic": None,
             "peak_source": "measured: rs_measure_int_peak, independent mad.lo.u32 chains on all %d SMs "
                            "(%.1f per clock per SM at the %.0f MHz maximum clock)"
                            % (pk["sms"], pk["mad_lo_u32"] / (pk["sms"] * pk["clock_max_mhz"] * 1e6),
@@ -324,8 +335,9 @@ def roofline(info, g1_ms, clk, kernel="G1 (reduce + evaluate + univariate result
 def whole_path_work(info, npairs, ms, peak):
     """Algorithmic modular products of one step by stage (a3 evaluation, a4
     univariate resultants, a5 interpolation counted in its direct
-    convolution form, a6 Garner digits) and the whole path's rate at 4 IMAD
-    per product against the same derived peak as the G1 roofline."""
+    convolution form, a6 Garner digits) and the whole path's rate at the
+    conventional 4 IMAD per product (products that share a reduction execute
+    fewer) against the same peak as the G1 roofline."""
     parts = {"eval": info["modmul_eval"], "prs": info["modmul_prs"], "interp": info["modmul_interp"],
              "crt": info["modmul_crt"]}
     total = sum(parts.values())
@@ -562,7 +574,7 @@ def batch_main(args, world, rank, local, dist):
     g1 = statistics.mean(stage["images"])
     if args.univariate == "schur":
         rf = roofline(info, g1, clk, "G1, Schur variant (reduce + evaluate + Schur on generators + "
-                                     "elimination fallback)")
+                                     "elimination fallback)", "schur")
     else:
         rf = roofline(info, g1, clk)
     if args.workload == "batch" and npairs == 512 and args.univariate == "prs":

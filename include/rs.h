@@ -196,7 +196,8 @@ typedef struct {
   double modmul_eval;         /* algorithmic modular products: evaluation (a3; the two images of
                                   a point pair +-x share one evaluation of the even and odd
                                   parts, plus one product per coefficient each) */
-  double modmul_prs;          /* univariate resultants (a4) */
+  double modmul_prs;          /* univariate resultants (a4): the products of the remainder sequence's
+                                  double steps (three per coefficient, with one reduction) */
   double modmul_interp;       /* interpolation (a5) */
   double modmul_crt;          /* Garner CRT (a6) */
   int64_t input_bytes;        /* host->device bytes of one upload */
